@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "gauge_pack.h"
+#include "sq_fixed.cuh"
 #include "serve.h"
 #include "sq_host.h"
 
@@ -34,6 +35,8 @@ LinkScales GaugeField::scales(int prec, int recon) const {
   s.long_k = long_scale / 32767.f;
   s.recon_d = (long_s != 0) ? 1.0 / long_s : 0.0;
   s.recon_f = (float)s.recon_d;
+  s.fixed = prec == PREC_F64 && fixed && (recon == 18 || f64_12_fixed);
+  s.fixed_exp = fixed_exp;
   if (prec == PREC_I16 && recon == 12) s.recon_f = (float)((double)s.long_k / long_s);
   return s;
 }
@@ -252,7 +255,7 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
     if (std::abs(det.imag()) > 1e-10 * std::abs(det) || gf->long_s == 0) gf->long_s = 0;
   }
   unsigned long long *stats_d = nullptr;
-  unsigned long long stats_h[3] = {0, 0, 0};
+  unsigned long long stats_h[4] = {0, 0, 0, 0};
   cudaError_t e = cudaMalloc(&stats_d, sizeof(stats_h));
   if (e == cudaSuccess) {
     cudaMemsetAsync(stats_d, 0, sizeof(stats_h), st);
@@ -267,10 +270,12 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
     if (tmp) cudaFree(tmp);
     return SQ_ERR_CUDA;
   }
-  double fmax_, lmax_, rerr;
+  double fmax_, lmax_, rerr, least;
   std::memcpy(&fmax_, &stats_h[0], 8);
   std::memcpy(&lmax_, &stats_h[1], 8);
   std::memcpy(&rerr, &stats_h[2], 8);
+  stats_h[3] = ~stats_h[3];
+  std::memcpy(&least, &stats_h[3], 8);
   if (!std::isfinite(fmax_) || !std::isfinite(lmax_)) {
     if (tmp) cudaFree(tmp);
     return SQ_ERR_NONFINITE;
@@ -278,7 +283,15 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
   gf->fat_scale = (float)fmax_;
   gf->long_scale = (float)lmax_;
   gf->recon12_ok = gf->long_s != 0 && rerr <= 1e-10 * std::abs(gf->long_s);
+  // Fixed-point FP64 links hold every element to 2^-56 of the field's largest:
+  // finer than FP64's own rounding of the mat-vecs while each direction's
+  // links reach 2^-4 of that largest element.  Fields with smaller links (or
+  // elements that are not finite) keep doubles and FP64 FMAs.
+  const double lmost = std::max(fmax_, lmax_);
+  if (lmost > 0) gf->fixed_exp = std::ilogb(lmost) + 1;
+  gf->fixed = lmost > 0 && least >= lmost / 16 && std::abs(gf->fixed_exp) <= 60;
   PackScales ps;
+  ps.to_fixed = gf->fixed ? std::ldexp(1.0, FX_BITS - gf->fixed_exp) : 0.0;
   ps.fat_inv = gf->fat_scale > 0 ? 32767.0f / gf->fat_scale : 0.f;
   ps.long_inv = gf->long_scale > 0 ? 32767.0f / gf->long_scale : 0.f;
 
@@ -289,6 +302,10 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
     if (prec == PREC_I16 && (flags & SQ_GAUGE_NO_I16)) continue;
     for (int recon : {18, 12}) {
       if (recon == 12 && (!gf->recon12_ok || (flags & SQ_GAUGE_NO_LONG12))) continue;
+      if (prec == PREC_F64 && recon == 12 && gf->fixed) {
+        gf->f64_12_fixed = true;
+        continue;
+      }
       size_t b = link_site_bytes(prec, recon) * g.stride;
       for (int par = 0; par < 2 && rc == SQ_OK; ++par) {
         rc = ctx->alloc(b, &gf->links[prec][recon == 12][par]);

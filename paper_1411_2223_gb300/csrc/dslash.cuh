@@ -34,6 +34,7 @@
 
 #include "sq_device.cuh"
 #include "cg_finish.cuh"
+#include "sq_fixed.cuh"
 
 namespace sq {
 
@@ -316,6 +317,162 @@ __device__ __forceinline__ void pair_hops(const DslashArgs &a, const LinkScales 
           mat_vec_acc(acc[r], m[h], v);
         }
       }
+    }
+  }
+}
+
+// ------------------------------------------------------ FP64, fixed point
+// The 16 hops of an output site with integer multiply-adds (sq_fixed.cuh).
+// The sums are kept relative to the exponent E of the largest neighbour
+// component seen so far, with a bit to spare, so that in a field of even size
+// only the first hop raises it.  One hop matrix is held at a time: 126
+// registers, four 128-thread blocks per SM.  Keeping the next hop's loads in
+// flight (168 registers, three blocks) was slower: 113 against 110 us for one
+// system at 20^3 x 64, 1120 against 999 us for 12.  Neighbours outside the fixed-point range
+// (infinities, NaN, magnitudes near the ends of FP64) send the site to
+// fixed_site_fp64.
+
+// Neighbour vector v of the FP64 operators; for a reliable update's the two
+// parts x64 (v) and xs (d).
+template <bool XS>
+__device__ __forceinline__ void fx_gather(const DslashArgs &a, int rhs, int S, int n,
+                                          Vec3<double> &v, Vec3<double> &d) {
+  v = SpinorIO<PREC_F64>::load(a.in + (size_t)rhs * a.in_fb, S, n);
+  if constexpr (XS) {
+    const char *fx = a.xs + (size_t)rhs * a.xs_fb;
+    if (a.xs_prec == PREC_F32) {
+      const Vec3<float> s = SpinorIO<PREC_F32>::load(fx, S, n);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d.c[c] = make_double2(fx_widen(s.c[c].x), fx_widen(s.c[c].y));
+    } else {
+      d = SpinorIO<PREC_F64>::load(fx, S, n);
+    }
+  }
+}
+
+// One site and system by FP64 FMAs, from the fixed-point links.
+template <int MODE>
+__device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs, double *out) {
+  const Geom &g = a.g;
+  const int S = g.stride;
+  const SiteCoords sc = site_coords(g, a.out_parity, i);
+  const char *in = a.in + (size_t)rhs * a.in_fb;
+  const char *fx = (a.xs != nullptr) ? a.xs + (size_t)rhs * a.xs_fb : nullptr;
+  const double unit = ldexp(1.0, a.ls.fixed_exp - FX_BITS);
+  double acc[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+  for (int k = 0; k < 16; ++k) {
+    const int mu = k >> 2, h = k & 3;
+    float f;
+    const int n = hop_index(g, sc, mu, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1), f);
+    f *= (h & 1) ? -eta_sign(sc, mu) : eta_sign(sc, mu);
+    const int4 *m = reinterpret_cast<const int4 *>(a.links) + (size_t)k * 9 * S + i;
+    const Vec3<double> v = gather_in<PREC_F64, MODE, double>(in, fx, a.xs_prec, S, n, f);
+#pragma unroll 1
+    for (int e = 0; e < 9; ++e) {
+      const int4 q = m[(size_t)e * S];
+      const double mr = ((double)q.y * (1 << FX_LOW) + (double)q.x) * unit;
+      const double mi = ((double)q.w * (1 << FX_LOW) + (double)q.z) * unit;
+      const int r = e / 3, c = e % 3;
+      const double2 w = c == 0 ? v.c[0] : c == 1 ? v.c[1] : v.c[2];
+      acc[2 * r] = fma(mr, w.x, fma(-mi, w.y, acc[2 * r]));
+      acc[2 * r + 1] = fma(mr, w.y, fma(mi, w.x, acc[2 * r + 1]));
+    }
+  }
+#pragma unroll 1
+  for (int c = 0; c < 6; ++c) out[c] = acc[c];
+}
+
+// XS: the input is x64 + xs (the reliable update's D_oe).
+template <int NR, int MODE, bool XS>
+__device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales &ls,
+                                           const SiteCoords &sc, int i, int r0,
+                                           const bool (&active)[NR], Vec3<double> (&acc)[NR]) {
+  const Geom &g = a.g;
+  const int S = g.stride;
+  const uint64_t pol = l2_link_policy(ls.keep);
+  FxAcc s[NR];
+  bool odd[NR];  // a neighbour outside the fixed-point range
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    fx_zero(s[r]);
+    odd[r] = false;
+  }
+  auto one = [&](int k, int nb, float f) {
+    int4 m[9];
+    const char *base = a.links + ((size_t)k * 9 * S + i) * 16;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const uint4 q = ld_stream_u4(base + (size_t)e * S * 16, pol);
+      m[e] = make_int4((int)q.x, (int)q.y, (int)q.z, (int)q.w);
+    }
+    const int sgn = f < 0.f ? -1 : 1;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (!active[r]) continue;
+      Vec3<double> v, d;
+      fx_gather<XS>(a, r0 + r, S, nb, v, d);
+      int e = fx_max_exponent(v);
+      if (XS) e = max(e, fx_max_exponent(d));
+      if (e >= s[r].E) {
+        if (e >= FX_MAX_E) {
+          odd[r] = true;
+          continue;
+        }
+        fx_raise(s[r], e + 1);
+      } else if (e < FX_MIN_E) {
+        odd[r] |= fx_any_nonzero(v) || (XS && fx_any_nonzero(d));
+        continue;
+      }
+      FxVec w;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        w.re[c] = fx_from_double(v.c[c].x, s[r].E, sgn);
+        w.im[c] = fx_from_double(v.c[c].y, s[r].E, sgn);
+      }
+      if (XS) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const Fx p = fx_from_double(d.c[c].x, s[r].E, sgn), q = fx_from_double(d.c[c].y, s[r].E, sgn);
+          const int lr = w.re[c].l + p.l, li = w.im[c].l + q.l;
+          w.re[c].h += p.h + (lr >> FX_LOW);
+          w.re[c].l = lr & FX_LOW_MASK;
+          w.im[c].h += q.h + (li >> FX_LOW);
+          w.im[c].l = li & FX_LOW_MASK;
+        }
+      }
+      fx_mat_vec(s[r], m, w);
+    }
+  };
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    const float eta = eta_sign(sc, mu);
+    float f;
+    int n = hop<+1>(g, sc, mu, f);
+    one(4 * mu, n, eta * f);
+    n = hop<-1>(g, sc, mu, f);
+    one(4 * mu + 1, n, -eta * f);
+    n = hop<+3>(g, sc, mu, f);
+    one(4 * mu + 2, n, eta * f);
+    n = hop<-3>(g, sc, mu, f);
+    one(4 * mu + 3, n, -eta * f);
+  }
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    // products are in units of 2^(fixed_exp - FX_BITS) 2^(E - 1022 - FX_BITS),
+    // the sums of 2^(2 FX_LOW) of these
+    const int ex = ls.fixed_exp + s[r].E - 1022 - 2 * FX_BITS + 2 * FX_LOW;
+    const double unit = __hiloint2double((ex + 1023) << 20, 0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[r].c[c].x = fx_to_double(s[r].hr[c], s[r].mr[c], unit);
+      acc[r].c[c].y = fx_to_double(s[r].hi[c], s[r].mi[c], unit);
+    }
+    if (active[r] && odd[r]) {
+      double o[6];
+      fixed_site_fp64<MODE>(a, i, r0 + r, o);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[r].c[c] = make_double2(o[2 * c], o[2 * c + 1]);
     }
   }
 }
@@ -671,9 +828,10 @@ inline size_t dslash_smem_bytes(int prec, int recon, int nr, int block) {
   return (size_t)npl * 16 * block;
 }
 
+// GATED: in dslash_gated_kernel, whose PLAIN form gathers x64 + xs.
 // One work item of the kernel: RHS tile blk % ntiles of the blockDim.x
 // sites from (blk / ntiles) * blockDim.x on.  A return ends the item.
-template <int PREC, int RECON, int NR, int MODE, int OUTP>
+template <int PREC, int RECON, int NR, int MODE, int OUTP, bool GATED>
 __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned blk) {
   using R = typename AccumType<PREC>::R;
   const Geom &g = a.g;
@@ -794,6 +952,8 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
     } else if constexpr (kStaged) {
       multi_hops<RECON, NR, MODE, kEarly>(a, ls, sc, i, r0, active, acc, dyn_smem, vbuf);
       if constexpr (EpiStage<MODE, RECON, NR>::V > 0) cp_async_wait<0>();
+    } else if constexpr (RECON == RECON_FIXED) {
+      fixed_hops<NR, MODE, GATED && MODE == MODE_PLAIN>(a, ls, sc, i, r0, active, acc);
     } else if constexpr (PREC == PREC_F64 && NR == 1) {
       pair_hops<PREC, RECON, NR, MODE>(a, ls, sc, i, r0, active, acc);
     } else {
@@ -1071,8 +1231,8 @@ __device__ __forceinline__ int nth_bit(unsigned long long m, int j) {
 template <int PREC, int RECON, int NR, int MODE, int OUTP>
 __global__ void __launch_bounds__(DslashBounds<PREC, NR>::threads,
                                   DslashBounds<PREC, NR>::min_blocks)
-dslash_kernel(const DslashArgs a) {
-  dslash_item<PREC, RECON, NR, MODE, OUTP>(a, blockIdx.x);
+dslash_kernel(const __grid_constant__ DslashArgs a) {
+  dslash_item<PREC, RECON, NR, MODE, OUTP, false>(a, blockIdx.x);
 }
 
 // Resident blocks per SM of the one-system gated kernels (up to 168
@@ -1090,14 +1250,14 @@ constexpr int GATED_BLOCKS_PER_SM = 3;
 template <int RECON, int NR, int MODE, int OUTP>
 __global__ void __launch_bounds__(DslashBounds<PREC_F64, NR>::threads,
                                   NR == 1 ? GATED_BLOCKS_PER_SM : DslashBounds<PREC_F64, NR>::min_blocks)
-dslash_gated_kernel(const DslashArgs a) {
+dslash_gated_kernel(const __grid_constant__ DslashArgs a) {
   griddep_wait();  // the gate reads what the previous kernel wrote
   const int ntiles = (a.nrhs + NR - 1) / NR;
   const unsigned long long act = active_tiles<NR>(a, ntiles);
   const int nact = __popcll(act);
   const int n = nact * ((a.g.vh + (int)blockDim.x - 1) / (int)blockDim.x);
   for (int k = blockIdx.x; k < n; k += gridDim.x)
-    dslash_item<PREC_F64, RECON, NR, MODE, OUTP>(a, (k / nact) * ntiles + nth_bit(act, k % nact));
+    dslash_item<PREC_F64, RECON, NR, MODE, OUTP, true>(a, (k / nact) * ntiles + nth_bit(act, k % nact));
   griddep_launch_dependents();
 }
 

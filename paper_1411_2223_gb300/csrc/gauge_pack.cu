@@ -3,6 +3,7 @@
 // hop-matrix planes for every precision and link format.
 #include "sq_device.cuh"
 #include "gauge_pack.h"
+#include "sq_fixed.cuh"
 
 namespace sq {
 
@@ -37,19 +38,26 @@ __device__ __forceinline__ void dagger(cd m[9]) {
 }
 
 __global__ void gauge_stats_kernel(const cd *fat, const cd *lng, long nlinks, double inv_s,
-                                   unsigned long long *out /* [fat max, long max, recon err] */) {
+                                   unsigned long long *out /* [fat max, long max, recon err, min] */) {
   long k = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  double fm = 0, lm = 0, err = 0;
+  double fm = 0, lm = 0, err = 0, least = __longlong_as_double(0x7ff0000000000000ll);
   for (; k < nlinks; k += (long)gridDim.x * blockDim.x) {
     const cd *f = fat + k * 9;
     const cd *l = lng + k * 9;
     cd w[9];
+    double pf = 0, pl = 0;
+    bool finite = true;
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-      fm = fmax(fm, fmax(fabs(f[e].x), fabs(f[e].y)));
+      const cd v = f[e];
+      pf = fmax(pf, fmax(fabs(v.x), fabs(v.y)));
       w[e] = l[e];
-      lm = fmax(lm, fmax(fabs(w[e].x), fabs(w[e].y)));
+      pl = fmax(pl, fmax(fabs(w[e].x), fabs(w[e].y)));
+      finite &= isfinite(v.x) && isfinite(v.y) && isfinite(w[e].x) && isfinite(w[e].y);
     }
+    fm = fmax(fm, pf);
+    lm = fmax(lm, pl);
+    least = fmin(least, finite ? fmax(pf, pl) : 0.0);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
@@ -62,6 +70,7 @@ __global__ void gauge_stats_kernel(const cd *fat, const cd *lng, long nlinks, do
   atomic_max_pos(out + 0, fm);
   atomic_max_pos(out + 1, lm);
   atomic_max_pos(out + 2, err);
+  atomicMax(out + 3, ~(unsigned long long)__double_as_longlong(least));
 }
 
 __device__ __forceinline__ uint32_t link_word(cd v, float inv) {
@@ -77,7 +86,19 @@ __device__ void store_pairs(char *links, int S, int i, int mu, const cd ff[9], c
   char *fat = links + (size_t)mu * LL::mu_bytes * S;
   char *lng = fat + (size_t)LL::fat_bytes * S;
   const int nl = (RECON == 18) ? 9 : 6;  // stored elements per long link
-  if constexpr (PREC == PREC_F64) {
+  if (PREC == PREC_F64 && RECON == 18 && ps.to_fixed != 0.0) {
+    int4 *pf = reinterpret_cast<int4 *>(fat), *pl = reinterpret_cast<int4 *>(lng);
+    auto word = [&](cd v) {
+      const int2 re = fx_link_word(v.x, ps.to_fixed), im = fx_link_word(v.y, ps.to_fixed);
+      return make_int4(re.x, re.y, im.x, im.y);
+    };
+    for (int k = 0; k < 9; ++k) {
+      pf[(size_t)k * S + i] = word(ff[k]);
+      pf[(size_t)(9 + k) * S + i] = word(fb[k]);
+      pl[(size_t)k * S + i] = word(lf[k]);
+      pl[(size_t)(9 + k) * S + i] = word(lb[k]);
+    }
+  } else if constexpr (PREC == PREC_F64) {
     double2 *pf = reinterpret_cast<double2 *>(fat);
     double2 *pl = reinterpret_cast<double2 *>(lng);
     for (int k = 0; k < 9; ++k) {

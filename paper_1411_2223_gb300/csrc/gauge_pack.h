@@ -10,12 +10,15 @@ namespace sq {
 struct PackScales {
   float fat_inv;   // 32767 / fat scale (FP32): 16-bit code = rint(v * fat_inv)
   float long_inv;  // 32767 / long scale
+  double to_fixed; // FP64, 18-real: link value -> fixed-point units; 0: stored as doubles
 };
 
 // Per-field maxima over nlinks = 4V links: out[0] = max |re|,|im| of fat,
 // out[1] = same for long, out[2] = max deviation of the long links' third row
-// from inv_s * conj(row0 x row1).  out holds non-negative doubles as u64 bits
-// and must be zeroed by the caller.
+// from inv_s * conj(row0 x row1), out[3] = the complement of the bits of the
+// smallest, over the (site, direction) pairs, of the larger of the pair's two
+// links' maxima (of 0 for a pair with an element that is not finite).  out
+// holds non-negative doubles as u64 bits and must be zeroed by the caller.
 int launch_gauge_stats(const double *fat, const double *lng, long nlinks, double inv_s,
                        unsigned long long *out, cudaStream_t st);
 

@@ -300,6 +300,9 @@ __device__ __forceinline__ Vec3<RO> convert(const Vec3<RI> &v) {
 //
 //   precision/recon   fat pair          long pair
 //   F64 / 18          18 x 16 B         18 x 16 B
+//                     (one complex element each: two doubles, or for a
+//                     field whose links allow it the two fixed-point pairs
+//                     of sq_fixed.cuh -- LinkScales::fixed)
 //   F64 / 12          18 x 16 B         12 x 16 B (rows 0, 1 of each)
 //   F32 / 18           9 x 16 B          9 x 16 B
 //   F32 / 12           9 x 16 B          6 x 16 B
@@ -310,6 +313,9 @@ __device__ __forceinline__ Vec3<RO> convert(const Vec3<RI> &v) {
 
 template <int PREC, int RECON> struct LinkLayout;
 
+// Link form of an FP64 kernel whose 18-real links are fixed-point words.
+constexpr int RECON_FIXED = 1;
+
 #define SQ_LAYOUT(P, RC, FAT16, FAT8, LONG16, LONG8)                              \
   template <> struct LinkLayout<P, RC> {                                          \
     static constexpr int fat16 = FAT16, fat8 = FAT8, long16 = LONG16, long8 = LONG8; \
@@ -319,6 +325,7 @@ template <int PREC, int RECON> struct LinkLayout;
     static constexpr int site_bytes = 4 * mu_bytes;                               \
   };
 SQ_LAYOUT(PREC_F64, 18, 18, 0, 18, 0)
+SQ_LAYOUT(PREC_F64, RECON_FIXED, 18, 0, 18, 0)
 SQ_LAYOUT(PREC_F64, 12, 18, 0, 12, 0)
 SQ_LAYOUT(PREC_F32, 18, 9, 0, 9, 0)
 SQ_LAYOUT(PREC_F32, 12, 9, 0, 6, 0)
@@ -333,6 +340,8 @@ struct LinkScales {
   float recon_f;    // 12-real: row2 = recon_f * conj(row0 x row1) in stored units
   double recon_d;   // same, FP64 kernels
   int keep;         // set in the kernel: links read again by a later tile
+  int fixed;        // F64, 18-real: the links are fixed-point words (sq_fixed.cuh)
+  int fixed_exp;    // ... of value word * 2^(fixed_exp - FX_BITS)
 };
 
 // Loader of the four hop matrices of direction mu at site i.

@@ -1,0 +1,153 @@
+// FP64 mat-vecs on the integer multiply-add units.
+//
+// GB300 issues 2 FP64 multiply-adds per clock and SM, but 64 32 x 32 -> 64 bit
+// integer multiply-adds (mad.wide.s32; measured 59 lanes per clock).  A real
+// number of a mat-vec is therefore held as a 55-bit fixed-point value in two
+// words,
+//   v = (h 2^27 + l) 2^(E - 55),   |h| <= 2^28, |l| < 2^27,
+// relative to an exponent E of its block (all links: one for the field;
+// colour vectors: one per output site, raised while its 16 neighbours are
+// read), and a product is three integer multiply-adds into two 64-bit sums,
+//   hi += ah bh,   mid += ah bl + al bh,
+// exact but for the term al bl (below 2^-54 of the blocks' scales).  The sums
+// over the 96 real products of an output component neither round nor
+// overflow:
+//   |hi| <= 96 2^56 < 2^63,  |mid| <= 96 (2^28 2^27 + 2^26 2^28) < 2^63
+// (the links' low words are balanced, |al| <= 2^26).  The result is rounded to
+// FP64 once; a chain of FP64 FMAs rounds at each of its 96 steps.  Against a
+// long-double Dslash of Gaussian vectors the 2-norm error is 1.5e-16, with
+// FP64 FMAs 3.5e-16 (2.7e-16 against 3.5e-16 where neighbouring sites differ
+// by factors up to e^8), the largest error of a component 5e-16 against 2e-15.
+//
+// What it bounds: the FP64 Dslash of one system at 20^3 x 64 went from
+// 321.6 us (FP64 units 100 % busy) to 110 us, 0.84 of the HBM rate for its
+// 2400 bytes per site; with 12 systems, where the links are read once, from
+// 3550 to 999 us (350 instructions per hop and system, 16 warps per SM: bound
+// by their latency).
+#pragma once
+
+#include "sq_device.cuh"
+
+namespace sq {
+
+constexpr int FX_LOW = 27;                 // bits of a low word
+constexpr int FX_BITS = 55;                // bits of a value
+constexpr int FX_LOW_MASK = (1 << FX_LOW) - 1;
+// Biased FP64 exponents the fixed-point path takes: below FX_MIN_E a vector
+// counts as zero at every scale in use, from FX_MAX_E on (which includes
+// infinities and NaN) the site is computed with FP64 FMAs.
+constexpr int FX_MIN_E = 128, FX_MAX_E = 1900;
+
+struct Fx { int h, l; };
+struct FxVec { Fx re[3], im[3]; };
+
+__device__ __forceinline__ int fx_hi_word(double v) { return __double2hiint(v); }
+
+// Largest biased exponent of a colour vector's six components.
+__device__ __forceinline__ int fx_max_exponent(const Vec3<double> &v) {
+  int m = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    m = max(m, fx_hi_word(v.c[c].x) & 0x7fffffff);
+    m = max(m, fx_hi_word(v.c[c].y) & 0x7fffffff);
+  }
+  return m >> 20;
+}
+__device__ __forceinline__ bool fx_any_nonzero(const Vec3<double> &v) {
+  int m = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    m |= (fx_hi_word(v.c[c].x) << 1) | __double2loint(v.c[c].x) | (fx_hi_word(v.c[c].y) << 1) |
+         __double2loint(v.c[c].y);
+  return m != 0;
+}
+
+// v (biased exponent <= E) as a fixed-point value relative to 2^(E - 1022),
+// times sgn (+1 or -1): the 53-bit mantissa, shifted up by 2 and down by the
+// distance of the exponents, the bits below the last one dropped.
+__device__ __forceinline__ Fx fx_from_double(double v, int E, int sgn) {
+  const unsigned H = (unsigned)__double2hiint(v), L = (unsigned)__double2loint(v);
+  const int d = E - (int)((H >> 20) & 0x7ff);
+  const unsigned mh = (H & 0xfffff) | 0x100000;
+  const unsigned Mh = __funnelshift_l(L, mh, 2);
+  unsigned Ml = __funnelshift_rc(L << 2, Mh, d);         // clamps at 32: then the high word
+  Ml = __funnelshift_rc(Ml, 0, max(d - 32, 0));
+  const unsigned Mr = __funnelshift_rc(Mh, 0, d);
+  const int s = ((int)H >> 31) ^ (sgn >> 31);            // 0 or -1
+  Fx o;
+  o.h = ((int)__funnelshift_l(Ml, Mr, 32 - FX_LOW) ^ s) - s;
+  o.l = ((int)(Ml & FX_LOW_MASK) ^ s) - s;
+  return o;
+}
+
+// FP32 value as the FP64 value of the same number without the conversion
+// unit; zero for zero and for FP32 denormals, infinities and NaN kept.
+__device__ __forceinline__ double fx_widen(float f) {
+  const unsigned b = __float_as_uint(f);
+  const unsigned e = (b >> 23) & 0xff;
+  unsigned E = e + 896;
+  E = (e == 255) ? 2047 : E;
+  const unsigned H = (b & 0x80000000u) | (E << 20) | ((b & 0x7fffff) >> 3);
+  return e == 0 ? 0.0 : __hiloint2double((int)H, (int)(b << 29));
+}
+
+__device__ __forceinline__ void fx_mac(long long &hi, long long &mid, const Fx a, const Fx b) {
+  hi += (long long)a.h * b.h;
+  mid += (long long)a.h * b.l;
+  mid += (long long)a.l * b.h;
+}
+
+struct FxAcc {
+  long long hr[3], mr[3], hi[3], mi[3];  // real part: hr, mr; imaginary part: hi, mi
+  int E;                                 // the vectors' exponent
+};
+
+__device__ __forceinline__ void fx_zero(FxAcc &a) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) a.hr[c] = a.mr[c] = a.hi[c] = a.mi[c] = 0;
+  a.E = FX_MIN_E;
+}
+
+// Raise the exponent of the sums to E.
+__device__ __forceinline__ void fx_raise(FxAcc &a, int E) {
+  const int s = min(E - a.E, 63);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    a.hr[c] >>= s; a.mr[c] >>= s;
+    a.hi[c] >>= s; a.mi[c] >>= s;
+  }
+  a.E = E;
+}
+
+// acc += M v, M given as 9 (re, im) pairs of fixed-point values
+__device__ __forceinline__ void fx_mat_vec(FxAcc &a, const int4 (&m)[9], const FxVec &v) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const Fx nim = {-v.im[c].h, -v.im[c].l};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int4 q = m[3 * r + c];
+      const Fx mr = {q.y, q.x}, mi = {q.w, q.z};
+      fx_mac(a.hr[r], a.mr[r], mr, v.re[c]);
+      fx_mac(a.hi[r], a.mi[r], mr, v.im[c]);
+      fx_mac(a.hr[r], a.mr[r], mi, nim);
+      fx_mac(a.hi[r], a.mi[r], mi, v.re[c]);
+    }
+  }
+}
+
+// (hi 2^27 + mid) 2^27 in units of the operands' last bits, times `unit`
+__device__ __forceinline__ double fx_to_double(long long hi, long long mid, double unit) {
+  const double d = (double)(hi + (mid >> FX_LOW));
+  const double r = (double)((int)mid & FX_LOW_MASK);
+  return fma(r, 1.0 / (1 << FX_LOW), d) * unit;
+}
+
+// Stored form of a link element: (re.l, re.h, im.l, im.h), low words balanced.
+__device__ __forceinline__ int2 fx_link_word(double v, double to_fixed) {
+  const long long q = __double2ll_rn(v * to_fixed);
+  const long long h = (q + (1ll << (FX_LOW - 1))) >> FX_LOW;
+  return make_int2((int)(q - (h << FX_LOW)), (int)h);
+}
+
+}  // namespace sq

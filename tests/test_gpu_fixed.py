@@ -1,0 +1,156 @@
+"""The FP64 operator on fixed-point links (csrc/sq_fixed.cuh).
+
+A 55-bit fixed-point mat-vec drops at most 2^-54 of the product of the two
+operands' scales per real product and rounds the sum of an output component
+to FP64 once (2^-53 relative).  For Gaussian vectors the largest of the 96
+neighbour components is about 4 times their RMS and the links' elements are
+at most 1.2, so an output component (RMS about 2 in those units) is off by
+at most about 10 * 2^-54 * 5 / 2 of its RMS in the dropped terms (random
+signs over 96 products): the 2-norm error stays below 2^-51.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from gpu_helpers import gauge, gpu_dslash, rel, site_rel
+
+pytestmark = pytest.mark.gpu
+
+DIMS = [(2, 4, 2, 6), (4, 6, 8, 10), (6, 4, 10, 4)]
+
+
+def _reference(dims, fat, lng, v_half, out_parity, t_sign=1):
+    """D v in long double (64 or more mantissa bits)."""
+    lx, ly, lz, lt = dims
+    vol = lx * ly * lz * lt
+    ld = np.clongdouble
+    full = np.zeros((vol, 3), dtype=ld)
+    full[oracle.half_sites(dims, 1 - out_parity)] = v_half
+    lex = np.arange(vol)
+    c = np.stack([lex % lx, (lex // lx) % ly, (lex // (lx * ly)) % lz, lex // (lx * ly * lz)], 1)
+    st = np.array([1, lx, lx * ly, lx * ly * lz])
+    out = np.zeros((vol, 3), dtype=ld)
+
+    def at(mu, d):
+        n = (c[:, mu] + d) % dims[mu]
+        wraps = np.floor_divide(c[:, mu] + d, dims[mu])
+        s = np.where((mu == 3) & (wraps % 2 != 0), t_sign, 1)
+        return lex + (n - c[:, mu]) * st[mu], s[:, None]
+
+    for mu in range(4):
+        eta = (1 - 2 * (c[:, :mu].sum(1) & 1))[:, None] * np.longdouble(0.5)
+        for u, d in ((fat, 1), (lng, 3)):
+            u = u[:, mu].astype(ld)
+            n, s = at(mu, d)
+            out += eta * s * (u * full[n][:, None, :]).sum(-1)
+            n, s = at(mu, -d)
+            out -= eta * s * (np.conj(np.swapaxes(u[n], 1, 2)) * full[n][:, None, :]).sum(-1)
+    return out[oracle.half_sites(dims, out_parity)]
+
+
+@pytest.mark.parametrize('dims', DIMS)
+@pytest.mark.parametrize('spread', [0, 8])
+def test_fixed_point_dslash_error(sq, dims, spread):
+    """Even fields, and sites whose magnitudes differ by up to e^16."""
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    rng = np.random.default_rng(4)
+    gid = sq.gauge_load(dims, fat, lng, antiperiodic_t=True)
+    try:
+        for p in (0, 1):
+            v = synth.gaussian_source(vh, 5 + p) * np.exp(rng.uniform(-spread, spread, (vh, 1)))
+            got = gpu_dslash(sq, gid, 'f64', 18, v, p, vh)
+            want = _reference(dims, fat, lng, v, p, t_sign=-1)
+            assert rel(got, want.astype(np.complex128)) <= 2.0 ** -51
+            assert site_rel(got, want.astype(np.complex128)) <= 2.0 ** -48
+    finally:
+        sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('scale', [1e-300, 1e-30, 1e250, 1e300])
+def test_magnitudes_at_the_ends_of_fp64(sq, scale):
+    """Inside and outside the fixed-point exponents; also a single non-zero
+    site (all other neighbours zero)."""
+    dims = (4, 6, 8, 10)
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    v = synth.gaussian_source(vh, 6)
+    point = np.zeros_like(v)
+    point[17] = v[17]
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        for w in (v, point):
+            got = gpu_dslash(sq, gid, 'f64', 18, w * scale, 1, vh) / scale
+            assert rel(got, oracle.dslash_half(dims, fat, lng, w, 1)) <= 1e-15
+    finally:
+        sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('bad', [np.nan, np.inf, -np.inf])
+def test_non_finite_neighbours(sq, bad):
+    """A site is non-finite exactly where one of its neighbours is; the
+    others are untouched."""
+    dims = (4, 6, 8, 10)
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    v = synth.gaussian_source(vh, 7)
+    mark = np.zeros_like(v)
+    mark[31] = 1.0
+    hit = np.abs(oracle.dslash_half(dims, fat, lng, mark, 1)).sum(1) > 0
+    want = oracle.dslash_half(dims, fat, lng, v, 1)
+    v[31, 1] = bad
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        got = gpu_dslash(sq, gid, 'f64', 18, v, 1, vh)
+        assert not np.isfinite(got[hit]).all(axis=1).any()
+        assert rel(got[~hit], want[~hit]) <= 1e-15
+    finally:
+        sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('least', [1.0, 2.0 ** -3, 2.0 ** -6, 0.0])
+def test_links_of_uneven_size(sq, least):
+    """Links much smaller than the field's largest keep FP64 FMAs: every
+    output site is accurate on its own scale either way."""
+    dims = (4, 4, 4, 6)
+    fat, lng = (a.copy() for a in gauge(dims))
+    s = np.ones(oracle.volume(dims))
+    s[::2] = least
+    fat *= s[:, None, None, None]
+    lng *= s[:, None, None, None]
+    vh = oracle.volume(dims) // 2
+    v = synth.gaussian_source(vh, 8)
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        for p in (0, 1):
+            got = gpu_dslash(sq, gid, 'f64', 18, v, p, vh)
+            want = oracle.dslash_half(dims, fat, lng, v, p)
+            assert rel(got, want) <= 1e-15
+            x = sq.cg_solve(gid, v, 0.3, 1e-10, precision='f64')[0]
+            assert oracle.true_residual(dims, fat, lng, 0.3, v, x) <= 1e-10
+    finally:
+        sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('nrhs', [2, 3, 4, 7])
+def test_tiles_give_the_bits_of_one_system(sq, nrhs):
+    """Every tile of systems computes what the one-system kernel does."""
+    import torch
+    dims = (4, 6, 8, 10)
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        nbytes, _ = sq.spinor_bytes(gid, 'f64')
+        src = torch.zeros((nrhs, nbytes), dtype=torch.uint8, device='cuda')
+        out, one = torch.zeros_like(src), torch.zeros_like(src)
+        for j in range(nrhs):
+            v = torch.from_numpy(synth.gaussian_source(vh, j)).cuda()
+            sq.pack_spinor(gid, 'f64', v, src[j])
+            sq.dslash_apply(gid, 0, 'f64', 18, src[j], one[j])
+        sq.dslash_apply_multi(gid, 0, 'f64', 18, nrhs, src, out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, one)
+    finally:
+        sq.gauge_free(gid)
