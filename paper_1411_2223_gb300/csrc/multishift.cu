@@ -255,6 +255,9 @@ int ms_work_get(sq_ctx *ctx, GaugeField *gf, int gid, int prec, int recon, int n
   SQ_CUDA_TRY(cudaMalloc((void **)&w->partial, sizes[9]));
   SQ_CUDA_TRY(cudaMalloc((void **)&w->counters, sizes[10]));
   SQ_CUDA_TRY(cudaMemset(w->counters, 0, sizes[10]));
+  // the clears are on the legacy stream, the solver's kernels on streams that
+  // do not wait for it
+  SQ_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
   SQ_CUDA_TRY(cudaMallocHost((void **)&w->bs_h, sizes[7]));
   SQ_CUDA_TRY(cudaMallocHost((void **)&w->sh_h, sizes[8]));
   *out = w.get();

@@ -78,6 +78,9 @@ int cg_work_create(sq_ctx *ctx, GaugeField *gf, int prec, int recon, int nrhs, C
   SQ_CUDA_TRY(cudaMemset(w->partial, 0, sizes[8]));
   // vectors start zeroed so no kernel reads NaN garbage from padding
   for (int k = 0; k < 7; ++k) SQ_CUDA_TRY(cudaMemset(*ptrs[k], 0, sizes[k]));
+  // the clears are on the legacy stream, the solver's kernels on streams that
+  // do not wait for it
+  SQ_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
   SQ_CUDA_TRY(cudaMallocHost((void **)&w->slots_h, sizes[7]));
   for (int k = 0; k < nrhs; ++k) {
     std::memset(&w->slots_h[k], 0, sizeof(SlotState));
