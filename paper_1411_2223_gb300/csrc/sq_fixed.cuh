@@ -1,7 +1,7 @@
 // FP64 mat-vecs on the integer multiply-add units.
 //
-// GB300 issues 2 FP64 multiply-adds per clock and SM, but 64 32 x 32 -> 64 bit
-// integer multiply-adds (mad.wide.s32; measured 59 lanes per clock).  A real
+// GB300 issues 2 FP64 multiply-adds per clock and SM, but 32 32 x 32 -> 64 bit
+// integer multiply-adds (mad.wide.s32).  A real
 // number of a mat-vec is therefore held as a 55-bit fixed-point value in two
 // words,
 //   v = (h 2^27 + l) 2^(E - 55),   |h| <= 2^28, |l| < 2^27,

@@ -146,3 +146,61 @@ def test_npr_arguments(sq):
 
 
 SQ_MAX = 16
+
+
+@pytest.mark.parametrize('nops', [1, 2, 3, 4, 5, 8, 9, 16, 17])
+def test_every_slicing_of_the_contraction(sq, nops):
+    """The number of operators picks how the sum over corners is split."""
+    dims = (4, 4, 6, 4)
+    links, props = _inputs(dims, seed=5)
+    ops = (OPS16 + [(2, 7, 1, 8)])[:nops]
+    out, hc = _gpu(sq, dims, links, props, ops)
+    want = oracle.npr_four_fermion(dims, links, props, ops)
+    _close(hc, want)
+    _close(out, want.sum(axis=0))
+
+
+@pytest.mark.parametrize('what', ['links3', 'links0.1', 'small', 'large', 'tiny', 'huge', 'spread',
+                                  'zero', 'equal'])
+def test_inputs_inside_and_outside_the_fixed_point_form(sq, what):
+    """Hypercubes that do not fit the two-word form go through FP64; either
+    way every hypercube holds the tolerance on its own scale.  'equal': all
+    terms of every sum equal, the largest sums the form can meet."""
+    dims = (4, 4, 6, 4)
+    links, props = _inputs(dims, seed=6)
+    if what == 'links3':
+        links = links * 3.0
+    elif what == 'links0.1':
+        links = links * 0.1
+    elif what in ('small', 'large', 'tiny', 'huge'):
+        s = {'small': 1e-40, 'large': 1e40, 'tiny': 1e-70, 'huge': 1e70}[what]
+        props = [p * s for p in props]
+    elif what == 'spread':  # hypercubes of very different size
+        s = np.exp(np.random.default_rng(2).uniform(-30, 30, props[0].shape[0]))[:, None, None]
+        props = [p * s for p in props]
+    elif what == 'zero':
+        props[2] = np.zeros_like(props[2])
+    elif what == 'equal':
+        links = snpr.unit_links(dims)
+        props = [np.full_like(p, 0.9999999 + 0.9999999j) for p in props]
+    ops = OPS16[:5] + [(0, 0, 0, 0)]
+    out, hc = _gpu(sq, dims, links, props, ops)
+    want = oracle.npr_four_fermion(dims, links, props, ops)
+    if what == 'zero':
+        assert np.all(hc == 0) and np.all(out == 0)
+        return
+    scale = np.abs(want).max(axis=tuple(range(1, want.ndim)), keepdims=True)
+    assert np.all(np.abs(hc - want) <= TOL * scale)
+    _close(out, want.sum(axis=0))
+
+
+@pytest.mark.parametrize('bad', [np.nan, np.inf])
+def test_non_finite_inputs_stay_in_their_hypercube(sq, bad):
+    dims = (4, 4, 6, 4)
+    links, props = _inputs(dims, seed=7)
+    want = oracle.npr_four_fermion(dims, links, props, OPS16[:3])
+    props[1] = props[1].copy()
+    props[1][0, 1, 2] = bad  # site 0: hypercube 0
+    _, hc = _gpu(sq, dims, links, props, OPS16[:3])
+    assert not np.isfinite(hc[0]).all()
+    _close(hc[1:], want[1:])
