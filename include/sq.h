@@ -184,8 +184,9 @@ int gauge_fatten(sq_ctx *ctx, const int dims[4], const double *thin_dev, double 
  * give 9/8 and -1/24 on unit links.  The paper's lattices are MILC asqtad
  * ensembles (Sec. 2, Fig. 1).  Arrays and `stream` as for gauge_fatten; the
  * paths are built as nested staple fields in a stream-ordered device scratch
- * of 288 bytes per site, taken and returned on `stream` (outside the HBM
- * budget). */
+ * of 2736 bytes per site, taken and returned on `stream` (outside the HBM
+ * budget); where the device refuses that much, the lattice is done in slabs of
+ * time slices with a part of it. */
 int gauge_fatten_asqtad(sq_ctx *ctx, const int dims[4], const double *thin_dev,
                         const double coeffs[6], double *fat_dev, double *lng_dev, void *stream);
 

@@ -91,10 +91,15 @@ __device__ __forceinline__ double fx_widen(float f) {
   return e == 0 ? 0.0 : __hiloint2double((int)H, (int)(b << 29));
 }
 
+// In PTX: written as 64-bit C++ products the compiler turns some of them (words
+// cut out of 64-bit values) into three instructions.
+__device__ __forceinline__ void fx_mac1(long long &s, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
+}
 __device__ __forceinline__ void fx_mac(long long &hi, long long &mid, const Fx a, const Fx b) {
-  hi += (long long)a.h * b.h;
-  mid += (long long)a.h * b.l;
-  mid += (long long)a.l * b.h;
+  fx_mac1(hi, a.h, b.h);
+  fx_mac1(mid, a.h, b.l);
+  fx_mac1(mid, a.l, b.h);
 }
 
 struct FxAcc {

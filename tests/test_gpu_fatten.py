@@ -121,3 +121,99 @@ def test_asqtad_full_size_20x64(sq):
     f0, l0 = oracle.asqtad_links(dims, thin)
     assert np.abs(fat.cpu().numpy() - f0).max() <= 1e-14
     assert np.abs(lng.cpu().numpy() - l0).max() <= 1e-15
+
+
+def _asqtad_ref(dims, u, coeffs):
+    """The path set as nested staples, on the CPU in complex128."""
+    one, three, five, seven, lepage, naik = coeffs
+    dag = lambda m: np.conj(np.swapaxes(m, -1, -2))  # noqa: E731
+    sh = lambda a, mu, d: synth.shift_field(a, dims, mu, d)  # noqa: E731
+
+    def staple(w, mu, nu, s):
+        un = u[:, nu]
+        if s > 0:
+            return un @ sh(w, nu, 1) @ dag(sh(un, mu, 1))
+        return sh(dag(un) @ w @ sh(un, mu, 1), nu, -1)
+
+    fat, lng = np.empty_like(u), np.empty_like(u)
+    for mu in range(4):
+        um = u[:, mu]
+        acc = one * um
+        for nu in range(4):
+            if nu == mu:
+                continue
+            for s in (-1, 1):
+                s3 = staple(um, mu, nu, s)
+                acc = acc + three * s3 + lepage * staple(s3, mu, nu, s)
+                for rho in range(4):
+                    if rho in (mu, nu):
+                        continue
+                    for t in (-1, 1):
+                        s5 = staple(s3, mu, rho, t)
+                        sg = 6 - mu - nu - rho
+                        acc = acc + five * s5 + seven * (staple(s5, mu, sg, -1) + staple(s5, mu, sg, 1))
+        fat[:, mu] = acc
+        lng[:, mu] = naik * (um @ sh(um, mu, 1) @ sh(um, mu, 2))
+    return fat, lng
+
+
+@pytest.mark.parametrize('what', ['su3', 'one', 'three', 'five', 'seven', 'lepage', 'naik', 'none',
+                                  'mixed', 'scaled', 'small', 'uneven', 'general', 'zero'])
+def test_asqtad_forms(sq, what):
+    """Each kind of path alone, coefficients of very different size, and
+    links that take the fixed-point kernels (even in size) or the FP64 ones.
+    60 products of 3 x 3 matrices nested 6 deep: errors of a few ulp of the
+    largest link."""
+    import torch
+    dims = (4, 2, 6, 4)
+    u = synth.thin_links(dims, 0.7, 3)
+    c = [5 / 8, 1 / 16, 1 / 64, 1 / 384, -1 / 16, -1 / 24]
+    kinds = ['one', 'three', 'five', 'seven', 'lepage', 'naik']
+    if what in kinds:
+        c = [1.5 if k == what else 0.0 for k in kinds]
+    elif what == 'none':
+        c = [0.0] * 6
+    elif what == 'mixed':
+        c = [1e-3, -1e5, 1e-8, 3.0, 1e2, 1e-30]
+    elif what == 'scaled':
+        u = u * 7.0
+    elif what == 'small':
+        u = u * 1e-25
+    elif what == 'uneven':
+        u = u * np.exp(np.random.default_rng(1).uniform(-6, 0, u.shape[:2]))[..., None, None]
+    elif what == 'general':
+        r = np.random.default_rng(2)
+        u = r.standard_normal(u.shape) + 1j * r.standard_normal(u.shape)
+    elif what == 'zero':
+        u = np.zeros_like(u)
+    t = torch.from_numpy(u).cuda()
+    fat, lng = torch.full_like(t, float('nan')), torch.full_like(t, float('nan'))
+    sq.gauge_fatten_asqtad(dims, t, fat, lng, c)
+    f0, l0 = _asqtad_ref(dims, u, c)
+    for got, want in ((fat.cpu().numpy(), f0), (lng.cpu().numpy(), l0)):
+        assert np.isfinite(got).all()
+        if np.abs(want).max() == 0:
+            assert np.all(got == 0)
+            continue
+        assert rel(got, want) <= 2e-15
+        assert np.abs(got - want).max() <= 1e-14 * np.abs(want).max()
+
+
+@pytest.mark.parametrize('bad', [np.nan, np.inf])
+def test_asqtad_non_finite_links(sq, bad):
+    """Only links near the bad one are lost."""
+    import torch
+    dims = (10, 8, 8, 8)
+    u = synth.thin_links(dims, 0.25, 4)
+    f0, l0 = _asqtad_ref(dims, u, sq.ASQTAD_COEFFS)
+    u[0, 0, 1, 1] = bad
+    t = torch.from_numpy(u).cuda()
+    fat, lng = torch.empty_like(t), torch.empty_like(t)
+    sq.gauge_fatten_asqtad(dims, t, fat, lng)
+    got = fat.cpu().numpy()
+    c = np.stack(np.unravel_index(np.arange(u.shape[0]), dims, order='F'), 1)
+    d = np.minimum(c, np.array(dims) - c)
+    far = (d.max(axis=1) > 3)
+    assert not np.isfinite(got[0, 0]).all()
+    assert np.abs(got[far] - f0[far]).max() <= 1e-14
+    assert np.abs(lng.cpu().numpy()[far] - l0[far]).max() <= 1e-15
