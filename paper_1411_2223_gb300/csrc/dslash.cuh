@@ -332,12 +332,26 @@ __device__ __forceinline__ void pair_hops(const DslashArgs &a, const LinkScales 
 // (infinities, NaN, magnitudes near the ends of FP64) send the site to
 // fixed_site_fp64.
 
-// Neighbour vector v of the FP64 operators; for a reliable update's the two
-// parts x64 (v) and xs (d).
-template <bool XS>
+// Input of the FP64 operators: packed half vectors, the reliable update's
+// x64 + xs, or a canonical whole-lattice vector [site_lex][colour].
+enum FixedIn { IN_HALF = 0, IN_XS = 1, IN_FULL = 2 };
+
+__device__ __forceinline__ Vec3<double> load_full(const char *base, int lex) {
+  const double2 *p = reinterpret_cast<const double2 *>(base) + (size_t)3 * lex;
+  Vec3<double> v;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) v.c[c] = __ldg(p + c);
+  return v;
+}
+
+// Neighbour vector v at n (half index, or site_lex for IN_FULL); of IN_XS the
+// two parts x64 (v) and xs (d).
+template <int IN>
 __device__ __forceinline__ void fx_gather(const DslashArgs &a, int rhs, int S, int n,
                                           Vec3<double> &v, Vec3<double> &d) {
-  v = SpinorIO<PREC_F64>::load(a.in + (size_t)rhs * a.in_fb, S, n);
+  constexpr bool XS = IN == IN_XS;
+  if constexpr (IN == IN_FULL) v = load_full(a.in, n);
+  else v = SpinorIO<PREC_F64>::load(a.in + (size_t)rhs * a.in_fb, S, n);
   if constexpr (XS) {
     const char *fx = a.xs + (size_t)rhs * a.xs_fb;
     if (a.xs_prec == PREC_F32) {
@@ -351,7 +365,7 @@ __device__ __forceinline__ void fx_gather(const DslashArgs &a, int rhs, int S, i
 }
 
 // One site and system by FP64 FMAs, from the fixed-point links.
-template <int MODE>
+template <int MODE, int IN>
 __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs, double *out) {
   const Geom &g = a.g;
   const int S = g.stride;
@@ -367,7 +381,16 @@ __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs
     const int n = hop_index(g, sc, mu, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1), f);
     f *= (h & 1) ? -eta_sign(sc, mu) : eta_sign(sc, mu);
     const int4 *m = reinterpret_cast<const int4 *>(a.links) + (size_t)k * 9 * S + i;
-    const Vec3<double> v = gather_in<PREC_F64, MODE, double>(in, fx, a.xs_prec, S, n, f);
+    Vec3<double> v;
+    if constexpr (IN == IN_FULL) {
+      // the neighbour's parity is the other one: its x has the parity bit that remains
+      const SiteCoords nc = site_coords(g, 1 - a.out_parity, n);
+      v = load_full(a.in, nc.lex);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) { v.c[c].x *= f; v.c[c].y *= f; }
+    } else {
+      v = gather_in<PREC_F64, MODE, double>(in, fx, a.xs_prec, S, n, f);
+    }
 #pragma unroll 1
     for (int e = 0; e < 9; ++e) {
       const int4 q = m[(size_t)e * S];
@@ -383,11 +406,11 @@ __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs
   for (int c = 0; c < 6; ++c) out[c] = acc[c];
 }
 
-// XS: the input is x64 + xs (the reliable update's D_oe).
-template <int NR, int MODE, bool XS>
+template <int NR, int MODE, int IN>
 __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales &ls,
                                            const SiteCoords &sc, int i, int r0,
                                            const bool (&active)[NR], Vec3<double> (&acc)[NR]) {
+  constexpr bool XS = IN == IN_XS;
   const Geom &g = a.g;
   const int S = g.stride;
   const uint64_t pol = l2_link_policy(ls.keep);
@@ -411,7 +434,7 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
     for (int r = 0; r < NR; ++r) {
       if (!active[r]) continue;
       Vec3<double> v, d;
-      fx_gather<XS>(a, r0 + r, S, nb, v, d);
+      fx_gather<IN>(a, r0 + r, S, nb, v, d);
       int e = fx_max_exponent(v);
       if (XS) e = max(e, fx_max_exponent(d));
       if (e >= s[r].E) {
@@ -447,14 +470,15 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
 #pragma unroll 1
   for (int mu = 0; mu < 4; ++mu) {
     const float eta = eta_sign(sc, mu);
+    auto to = [](int lex) { return IN == IN_FULL ? lex : lex >> 1; };
     float f;
-    int n = hop<+1>(g, sc, mu, f);
+    int n = to(hop_lex<+1>(g, sc, mu, f));
     one(4 * mu, n, eta * f);
-    n = hop<-1>(g, sc, mu, f);
+    n = to(hop_lex<-1>(g, sc, mu, f));
     one(4 * mu + 1, n, -eta * f);
-    n = hop<+3>(g, sc, mu, f);
+    n = to(hop_lex<+3>(g, sc, mu, f));
     one(4 * mu + 2, n, eta * f);
-    n = hop<-3>(g, sc, mu, f);
+    n = to(hop_lex<-3>(g, sc, mu, f));
     one(4 * mu + 3, n, -eta * f);
   }
 #pragma unroll
@@ -470,7 +494,7 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
     }
     if (active[r] && odd[r]) {
       double o[6];
-      fixed_site_fp64<MODE>(a, i, r0 + r, o);
+      fixed_site_fp64<MODE, IN>(a, i, r0 + r, o);
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[r].c[c] = make_double2(o[2 * c], o[2 * c + 1]);
     }
@@ -953,7 +977,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
       multi_hops<RECON, NR, MODE, kEarly>(a, ls, sc, i, r0, active, acc, dyn_smem, vbuf);
       if constexpr (EpiStage<MODE, RECON, NR>::V > 0) cp_async_wait<0>();
     } else if constexpr (RECON == RECON_FIXED) {
-      fixed_hops<NR, MODE, GATED && MODE == MODE_PLAIN>(a, ls, sc, i, r0, active, acc);
+      fixed_hops<NR, MODE, GATED && MODE == MODE_PLAIN ? IN_XS : IN_HALF>(a, ls, sc, i, r0, active, acc);
     } else if constexpr (PREC == PREC_F64 && NR == 1) {
       pair_hops<PREC, RECON, NR, MODE>(a, ls, sc, i, r0, active, acc);
     } else {

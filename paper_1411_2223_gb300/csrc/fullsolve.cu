@@ -51,6 +51,29 @@ __global__ void half_to_full_kernel(Geom g, int parity, const char *half, double
   for (int k = 0; k < 3; ++k) c[k] = v.c[k];
 }
 
+// out = (m + D) in at the sites of one parity, on canonical whole-lattice
+// vectors: the neighbours are gathered from the caller's array and the result
+// goes straight to his, so the operator is two independent launches (the
+// second starts while the first drains) without scratch.
+// 14 x 18 x 22 x 54: 568 us with FP64 FMAs, 323 us with the fixed-point Dslash
+// on packed halves (split, two Dslash, two axpys, merge; scratch allocated and
+// freed per call), 138 us here, of which the links are 103 us of HBM time.
+__global__ void __launch_bounds__(128, 4) dirac_fixed_kernel(const __grid_constant__ DslashArgs a,
+                                                             double mass) {
+  griddep_launch_dependents();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= a.g.vh) return;
+  const SiteCoords sc = site_coords(a.g, a.out_parity, i);
+  const bool active[1] = {true};
+  Vec3<double> acc[1];
+  fixed_hops<1, MODE_PLAIN, IN_FULL>(a, a.ls, sc, i, 0, active, acc);
+  const Vec3<double> v = load_full(a.in, sc.lex);
+  double2 *o = reinterpret_cast<double2 *>(a.out) + (size_t)3 * sc.lex;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    o[c] = make_double2(fma(mass, v.c[c].x, 0.5 * acc[0].c[c].x), fma(mass, v.c[c].y, 0.5 * acc[0].c[c].y));
+}
+
 // out = a x + b y + c z on packed halves of precision P (z may be null)
 template <int P>
 __global__ void lincomb_kernel(Geom g, double a, const char *x, double b, const char *y, double c,
@@ -373,6 +396,26 @@ extern "C" int dirac_apply(sq_ctx *ctx, int gauge_id, double mass, const double 
   if (!gf->has(PREC_F64, 18)) return SQ_ERR_UNSUPPORTED;
   cudaSetDevice(ctx->device);
   const Geom &g = gf->g;
+  if (gf->fixed) {  // on the caller's own stream
+    cudaStream_t cs = stream ? (cudaStream_t)stream : cudaStreamLegacy;
+    DslashArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.g = g;
+    a.links = gf->link_ptr(PREC_F64, 18, 0);
+    a.ls = gf->scales(PREC_F64, 18);
+    a.in = reinterpret_cast<const char *>(in_dev);
+    a.out = reinterpret_cast<char *>(out_dev);
+    a.nrhs = 1;
+    const dim3 grid((g.vh + 127) / 128), block(128);
+    dirac_fixed_kernel<<<grid, block, 0, cs>>>(a, mass);
+    SQ_CUDA_TRY(cudaGetLastError());
+    a.out_parity = 1;
+    a.links = gf->link_ptr(PREC_F64, 18, 1);
+    SQ_CUDA_TRY(launch_pdl(dirac_fixed_kernel, grid, block, 0, cs, a, mass));
+    ctx->launches += 2;
+    SQ_CUDA_TRY(cudaStreamSynchronize(cs));
+    return SQ_OK;
+  }
   cudaStream_t st = pick_stream(ctx, stream);
   if (st == ctx->stream)  // a default stream (NULL: the legacy one): its work first
     SQ_CUDA_TRY(cudaStreamSynchronize(stream ? (cudaStream_t)stream : cudaStreamLegacy));

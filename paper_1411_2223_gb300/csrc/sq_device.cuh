@@ -53,9 +53,10 @@ __device__ __forceinline__ int hop_index(const Geom &g, const SiteCoords &s, int
 }
 
 // Same as hop_index for a hop length D known at compile time (|D| <= 3,
-// L >= 2: at most two wraps, only in the direction of the hop).
+// L >= 2: at most two wraps, only in the direction of the hop); hop_lex: the
+// neighbour's site_lex.
 template <int D>
-__device__ __forceinline__ int hop(const Geom &g, const SiteCoords &s, int mu, float &sign) {
+__device__ __forceinline__ int hop_lex(const Geom &g, const SiteCoords &s, int mu, float &sign) {
   const int L = g.L[mu];
   int c = s.c[mu] + D;
   bool w1, w2 = false;
@@ -69,7 +70,11 @@ __device__ __forceinline__ int hop(const Geom &g, const SiteCoords &s, int mu, f
     if constexpr (D < -1) { w2 = c < 0; c += w2 ? L : 0; }
   }
   sign = (mu == 3 && g.t_antiperiodic && (w1 != w2)) ? -1.f : 1.f;
-  return (s.lex + (c - s.c[mu]) * g.st[mu]) >> 1;
+  return s.lex + (c - s.c[mu]) * g.st[mu];
+}
+template <int D>
+__device__ __forceinline__ int hop(const Geom &g, const SiteCoords &s, int mu, float &sign) {
+  return hop_lex<D>(g, s, mu, sign) >> 1;
 }
 
 // eta_mu(x) = (-1)^(x_0 + ... + x_{mu-1})

@@ -13,7 +13,7 @@ import pytest
 
 import oracle
 import synth
-from gpu_helpers import gauge, gpu_dslash, rel, site_rel
+from gpu_helpers import gauge, gpu_dslash, rel, site_rel, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -154,3 +154,38 @@ def test_tiles_give_the_bits_of_one_system(sq, nrhs):
         assert torch.equal(out, one)
     finally:
         sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('dims', [(2, 2, 2, 2), (4, 6, 8, 10), (6, 2, 10, 4)])
+@pytest.mark.parametrize('antiperiodic', [False, True])
+def test_dirac_apply_gathers_from_the_whole_lattice(sq, dims, antiperiodic):
+    """Against the Dslash of the halves, on a side stream; with a site that
+    takes the FP64 form (its neighbours are infinite) and links that do."""
+    import torch
+    fat, lng = gauge(dims)
+    vol = oracle.volume(dims)
+    even, odd = oracle.half_sites(dims, 0), oracle.half_sites(dims, 1)
+    for scale in (1.0, 0.01):  # uneven links keep FP64 FMAs
+        f, l = fat.copy(), lng.copy()
+        f[0] *= scale
+        l[0] *= scale
+        gid = sq.gauge_load(dims, f, l, antiperiodic_t=antiperiodic)
+        try:
+            v = synth.gaussian_source(vol, 9)
+            want = np.empty_like(v)
+            for p, (a, b) in enumerate(((even, odd), (odd, even))):
+                want[a] = 0.07 * v[a] + gpu_dslash(sq, gid, 'f64', 18, v[b], p, vol // 2)
+            st = torch.cuda.Stream()
+            x = to_dev(v)
+            out = torch.full_like(x, float('nan'))
+            torch.cuda.synchronize()
+            sq.dirac_apply(gid, 0.07, x, out, stream=st)
+            assert rel(out.cpu().numpy(), want) <= 1e-15
+            v[even[0]] = np.inf
+            sq.dirac_apply(gid, 0.07, to_dev(v), out)
+            got = out.cpu().numpy()
+            bad = ~np.isfinite(got).all(axis=1)
+            assert bad[even[0]] and bad[odd].any() and not bad[even[1:]].any()
+            assert rel(got[~bad], want[~bad]) <= 1e-15
+        finally:
+            sq.gauge_free(gid)
