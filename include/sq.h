@@ -116,7 +116,10 @@ typedef struct {
     /* Launch shapes of the CG's two sloppy Dslash kernels as launched (the
      * tuner's choice, or a SQ_TUNE_CACHE entry): threads per block and
      * right-hand sides per thread of the D_oe kernel (with the reduction)
-     * and of the D_eo kernel (with the update).  0 where no batched CG ran. */
+     * and of the D_eo kernel (with the update).  A single system on a lattice of
+     * up to 512 sites per parity and SM runs as one resident kernel instead,
+     * unless a SQ_TUNE_CACHE entry gives these shapes: then its threads per
+     * block and 1.  0 where no batched CG ran. */
     int oe_block, oe_rhs_tile, eo_block, eo_rhs_tile;
 } sq_cg_stats;
 

@@ -570,8 +570,14 @@ int solve_batch_locked(sq_ctx *ctx, int gauge_id, int nrhs, const double *src,
   if (!w) {
     int rc = cg_work_create(ctx, gf, o.precision, o.long_recon, nrhs, &w);
     if (rc) return rc;
-    w->cfg_norm = tuned_dslash(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_NORM, st);
-    w->cfg_update = tuned_dslash(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_UPDATE, st);
+    // launch shapes that a tuning file gives are launched
+    if (!tuned_pinned(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_NORM) &&
+        !tuned_pinned(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_UPDATE))
+      w->resident_block = cg_resident_block(w);
+    if (!w->resident_block) {
+      w->cfg_norm = tuned_dslash(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_NORM, st);
+      w->cfg_update = tuned_dslash(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_UPDATE, st);
+    }
     w->cfg_ru_plain = tuned_dslash(ctx, *gf, PREC_F64, 18, nrhs, MODE_PLAIN, st);
     w->cfg_ru_resid = w->cfg_ru_plain;
     std::lock_guard<std::mutex> lk(g_cache_mu);
@@ -603,8 +609,14 @@ int solve_batch_locked(sq_ctx *ctx, int gauge_id, int nrhs, const double *src,
   for (int k = 0; k < nrhs; ++k) cg_slot_setup(w, k, masses[k], tol, o.delta, o.max_iter);
   int rc;
   if ((rc = cg_slots_upload(w, st))) return rc;
-  if ((rc = cg_enqueue_init(w, guess ? 1 : 0, st))) return rc;
-  if ((rc = cg_run(w, o.block_iters, !(o.flags & SQ_CG_NO_GRAPH), st))) return rc;
+  if (w->resident_block) {
+    // it begins with p = a r + beta p, which the start leaves due (a = 1, beta = 0)
+    if ((rc = cg_enqueue_init(w, guess ? 1 : 0, st, false))) return rc;
+    if ((rc = cg_run_resident(w, st))) return rc;
+  } else {
+    if ((rc = cg_enqueue_init(w, guess ? 1 : 0, st))) return rc;
+    if ((rc = cg_run(w, o.block_iters, !(o.flags & SQ_CG_NO_GRAPH), st))) return rc;
+  }
   if (launch_unpack(PREC_F64, gf->g, w->x64, w->f64_fb, cx, vec_elems, nrhs, st)) return SQ_ERR_ARG;
   ctx->launches++;
   if (!dev) SQ_CUDA_TRY(cudaMemcpyAsync(x, cx, canon_bytes, cudaMemcpyDeviceToHost, st));

@@ -218,6 +218,49 @@ __device__ __forceinline__ Vec3<float> i16_vector(const uint4 q, float f) {
   return v;
 }
 
+// acc_r += the four hops of direction mu, its link words in w.
+template <int RECON, int NR, bool CO>
+__device__ __forceinline__ void i16_dir(const DslashArgs &a, const LinkScales &ls, const SiteCoords &sc,
+                                        int mu, const uint32_t *w, int r0, const bool (&active)[NR],
+                                        Vec3<float> (&acc)[NR]) {
+  const Geom &g = a.g;
+  int nb[4];
+  float f[4];
+  nb[0] = hop<+1>(g, sc, mu, f[0]);
+  nb[1] = hop<-1>(g, sc, mu, f[1]);
+  nb[2] = hop<+3>(g, sc, mu, f[2]);
+  nb[3] = hop<-3>(g, sc, mu, f[3]);
+  const float eta = eta_sign(sc, mu);
+  const float kf = eta * ls.fat_k, kl = eta * ls.long_k;
+  f[0] *= kf;
+  f[1] *= -kf;
+  f[2] *= kl;
+  f[3] *= -kl;
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    if (!active[r]) continue;
+    const uint4 *in = reinterpret_cast<const uint4 *>(a.in + (size_t)(r0 + r) * a.in_fb);
+    uint4 q[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) q[h] = ld_field<CO>(in + nb[h]);
+    mat_vec_words(acc[r], w, i16_vector(q[0], f[0]));
+    mat_vec_words(acc[r], w + 9, i16_vector(q[1], f[1]));
+    if constexpr (RECON == 18) {
+      mat_vec_words(acc[r], w + 18, i16_vector(q[2], f[2]));
+      mat_vec_words(acc[r], w + 27, i16_vector(q[3], f[3]));
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        Mat3<float> m;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) m.e[e] = decode_word(w[18 + 6 * h + e]);
+        reconstruct_row2(m, ls.recon_f);
+        mat_vec_acc(acc[r], m, i16_vector(q[2 + h], f[2 + h]));
+      }
+    }
+  }
+}
+
 // buf holds direction 0's words on entry (loaded by the caller before the
 // kernel waited for its predecessor); each later direction's words are
 // loaded at its top.  Measured against keeping the next direction's words
@@ -229,47 +272,10 @@ __device__ __forceinline__ void i16_hops(const DslashArgs &a, const LinkScales &
                                          const SiteCoords &sc, int i, int r0,
                                          const bool (&active)[NR], Vec3<float> (&acc)[NR],
                                          I16Words<RECON> &buf) {
-  const Geom &g = a.g;
-  const int S = g.stride;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
-    if (mu > 0) i16_load_words<RECON>(a.links, S, i, mu, buf, ls.keep);
-    const uint32_t *w = buf.w;
-    int nb[4];
-    float f[4];
-    nb[0] = hop<+1>(g, sc, mu, f[0]);
-    nb[1] = hop<-1>(g, sc, mu, f[1]);
-    nb[2] = hop<+3>(g, sc, mu, f[2]);
-    nb[3] = hop<-3>(g, sc, mu, f[3]);
-    const float eta = eta_sign(sc, mu);
-    const float kf = eta * ls.fat_k, kl = eta * ls.long_k;
-    f[0] *= kf;
-    f[1] *= -kf;
-    f[2] *= kl;
-    f[3] *= -kl;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      if (!active[r]) continue;
-      const uint4 *in = reinterpret_cast<const uint4 *>(a.in + (size_t)(r0 + r) * a.in_fb);
-      uint4 q[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h) q[h] = __ldg(in + nb[h]);
-      mat_vec_words(acc[r], w, i16_vector(q[0], f[0]));
-      mat_vec_words(acc[r], w + 9, i16_vector(q[1], f[1]));
-      if constexpr (RECON == 18) {
-        mat_vec_words(acc[r], w + 18, i16_vector(q[2], f[2]));
-        mat_vec_words(acc[r], w + 27, i16_vector(q[3], f[3]));
-      } else {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          Mat3<float> m;
-#pragma unroll
-          for (int e = 0; e < 6; ++e) m.e[e] = decode_word(w[18 + 6 * h + e]);
-          reconstruct_row2(m, ls.recon_f);
-          mat_vec_acc(acc[r], m, i16_vector(q[2 + h], f[2 + h]));
-        }
-      }
-    }
+    if (mu > 0) i16_load_words<RECON>(a.links, a.g.stride, i, mu, buf, ls.keep);
+    i16_dir<RECON, NR, false>(a, ls, sc, mu, buf.w, r0, active, acc);
   }
 }
 
@@ -334,7 +340,8 @@ __device__ __forceinline__ void pair_hops(const DslashArgs &a, const LinkScales 
 
 // Input of the FP64 operators: packed half vectors, the reliable update's
 // x64 + xs, or a canonical whole-lattice vector [site_lex][colour].
-enum FixedIn { IN_HALF = 0, IN_XS = 1, IN_FULL = 2 };
+// IN_CO: packed half vectors by coherent loads (the resident CG).
+enum FixedIn { IN_HALF = 0, IN_XS = 1, IN_FULL = 2, IN_CO = 3 };
 
 __device__ __forceinline__ Vec3<double> load_full(const char *base, int lex) {
   const double2 *p = reinterpret_cast<const double2 *>(base) + (size_t)3 * lex;
@@ -351,7 +358,7 @@ __device__ __forceinline__ void fx_gather(const DslashArgs &a, int rhs, int S, i
                                           Vec3<double> &v, Vec3<double> &d) {
   constexpr bool XS = IN == IN_XS;
   if constexpr (IN == IN_FULL) v = load_full(a.in, n);
-  else v = SpinorIO<PREC_F64>::load(a.in + (size_t)rhs * a.in_fb, S, n);
+  else v = SpinorIO<PREC_F64>::template load<IN == IN_CO>(a.in + (size_t)rhs * a.in_fb, S, n);
   if constexpr (XS) {
     const char *fx = a.xs + (size_t)rhs * a.xs_fb;
     if (a.xs_prec == PREC_F32) {
@@ -388,6 +395,10 @@ __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs
       v = load_full(a.in, nc.lex);
 #pragma unroll
       for (int c = 0; c < 3; ++c) { v.c[c].x *= f; v.c[c].y *= f; }
+    } else if constexpr (IN == IN_CO) {
+      v = SpinorIO<PREC_F64>::template load<true>(in, S, n);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) { v.c[c].x *= f; v.c[c].y *= f; }
     } else {
       v = gather_in<PREC_F64, MODE, double>(in, fx, a.xs_prec, S, n, f);
     }
@@ -406,10 +417,13 @@ __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs
   for (int c = 0; c < 6; ++c) out[c] = acc[c];
 }
 
+// Directions mu0, mu0 + step, ...; with step > 1 `odd_site` says that a
+// neighbour was outside the range, and the caller has the site recomputed.
 template <int NR, int MODE, int IN>
 __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales &ls,
                                            const SiteCoords &sc, int i, int r0,
-                                           const bool (&active)[NR], Vec3<double> (&acc)[NR]) {
+                                           const bool (&active)[NR], Vec3<double> (&acc)[NR],
+                                           int mu0 = 0, int step = 1, bool *odd_site = nullptr) {
   constexpr bool XS = IN == IN_XS;
   const Geom &g = a.g;
   const int S = g.stride;
@@ -468,7 +482,7 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
     }
   };
 #pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) {
+  for (int mu = mu0; mu < 4; mu += step) {
     const float eta = eta_sign(sc, mu);
     auto to = [](int lex) { return IN == IN_FULL ? lex : lex >> 1; };
     float f;
@@ -492,7 +506,9 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
       acc[r].c[c].x = fx_to_double(s[r].hr[c], s[r].mr[c], unit);
       acc[r].c[c].y = fx_to_double(s[r].hi[c], s[r].mi[c], unit);
     }
-    if (active[r] && odd[r]) {
+    if (odd_site != nullptr) {
+      *odd_site = odd[r];
+    } else if (active[r] && odd[r]) {
       double o[6];
       fixed_site_fp64<MODE, IN>(a, i, r0 + r, o);
 #pragma unroll

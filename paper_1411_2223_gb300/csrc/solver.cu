@@ -20,6 +20,9 @@
 // wasted.  k iterations are captured once into a CUDA graph and replayed; the
 // host reads the slot states after each replay.  Finished slots make every
 // kernel skip their work, so overshooting the last block costs launches only.
+//
+// A single system on a small lattice runs the same iteration inside one
+// resident kernel (cg_resident.cu), which returns for the reliable updates.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -33,7 +36,7 @@ CGWork::~CGWork() {
   if (exec) cudaGraphExecDestroy(exec);
   if (slots_h) cudaFreeHost(slots_h);
   if (ctx) {
-    void *bufs[] = {x64, b64, t64, r, p, t, xs, slots_d, partial, counters};
+    void *bufs[] = {x64, b64, t64, r, p, t, xs, slots_d, partial, counters, resident};
     for (void *b : bufs)
       if (b) cudaFree(b);
     std::lock_guard<std::mutex> lk(ctx->mu);
@@ -59,7 +62,7 @@ int cg_work_create(sq_ctx *ctx, GaugeField *gf, int prec, int recon, int nrhs, C
   size_t sizes[] = {w->f64_fb * nrhs, w->f64_fb * nrhs, w->f64_fb * nrhs, w->fb * nrhs,
                     w->fb * nrhs,     w->fb * nrhs,     w->xs_fb * nrhs,
                     sizeof(SlotState) * nrhs, sizeof(double) * 4 * w->partial_stride,
-                    sizeof(unsigned) * 4 * w->counter_stride};
+                    sizeof(unsigned) * 4 * w->counter_stride, nrhs == 1 ? cg_resident_bytes(ctx, w->fb) : 256};
   char **ptrs[] = {&w->x64, &w->b64, &w->t64, &w->r, &w->p, &w->t, &w->xs};
   size_t total = 0;
   for (size_t s : sizes) total += s;
@@ -74,6 +77,8 @@ int cg_work_create(sq_ctx *ctx, GaugeField *gf, int prec, int recon, int nrhs, C
   SQ_CUDA_TRY(cudaMalloc((void **)&w->slots_d, sizes[7]));
   SQ_CUDA_TRY(cudaMalloc((void **)&w->partial, sizes[8]));
   SQ_CUDA_TRY(cudaMalloc((void **)&w->counters, sizes[9]));
+  SQ_CUDA_TRY(cudaMalloc(&w->resident, sizes[10]));
+  SQ_CUDA_TRY(cudaMemset(w->resident, 0, sizes[10]));
   SQ_CUDA_TRY(cudaMemset(w->counters, 0, sizes[9]));
   SQ_CUDA_TRY(cudaMemset(w->partial, 0, sizes[8]));
   // vectors start zeroed so no kernel reads NaN garbage from padding
@@ -155,13 +160,13 @@ static int check_launch(sq_ctx *ctx, int rc, int nkernels = 1) {
   return SQ_OK;
 }
 
-int cg_enqueue_init(CGWork *w, int guess, cudaStream_t st) {
+int cg_enqueue_init(CGWork *w, int guess, cudaStream_t st, bool xpay) {
   VecArgs va = vec_args(w, 3);
   int rc = check_launch(w->ctx, launch_cg_init(w->prec, va, guess, st));
   if (rc) return rc;
   if (guess) {
     if ((rc = cg_enqueue_ru(w, st))) return rc;
-    if ((rc = cg_enqueue_xpay(w, st))) return rc;
+    if (xpay && (rc = cg_enqueue_xpay(w, st))) return rc;
   }
   return SQ_OK;
 }
@@ -214,9 +219,8 @@ int cg_enqueue_xpay(CGWork *w, cudaStream_t st) {
   return check_launch(w->ctx, launch_cg_xpay(w->prec, vec_args(w, 1), st));
 }
 
-int cg_enqueue_iteration(CGWork *w, cudaStream_t st, int checkpoint) {
-  int rc;
-  // t = D_oe p, with |t|^2 + m^2 |p|^2 = <p, A p>: alpha
+// t = D_oe p, with |t|^2 + m^2 |p|^2 = <p, A p>
+static DslashArgs norm_args(CGWork *w) {
   DslashArgs a = dslash_args(w, w->prec, w->recon, 1);
   a.in = w->p;
   a.in_fb = w->fb;
@@ -225,11 +229,11 @@ int cg_enqueue_iteration(CGWork *w, cudaStream_t st, int checkpoint) {
   a.partial = w->partial;
   a.counter = w->counters;
   a.gate = GATE_RUNNING;
-  rc = check_launch(w->ctx, launch_dslash(w->prec, w->recon, w->cfg_norm.nr, MODE_NORM,
-                                          w->prec, a, w->cfg_norm.block, st));
-  if (rc) return rc;
-  if ((rc = check_launch(w->ctx, launch_cg_finish(0, vec_args(w, 0), st)))) return rc;
-  // Ap = m^2 p - D_eo t in registers: xs += alpha p, r -= alpha Ap, |r|^2: beta
+  return a;
+}
+
+// Ap = m^2 p - D_eo t in registers: xs += alpha p, r -= alpha Ap, |r|^2
+static DslashArgs update_args(CGWork *w) {
   DslashArgs b = dslash_args(w, w->prec, w->recon, 0);
   b.in = w->t;
   b.in_fb = w->fb;
@@ -243,6 +247,17 @@ int cg_enqueue_iteration(CGWork *w, cudaStream_t st, int checkpoint) {
   b.partial = w->partial + w->partial_stride;
   b.counter = w->counters + w->counter_stride;
   b.gate = GATE_RUNNING;
+  return b;
+}
+
+int cg_enqueue_iteration(CGWork *w, cudaStream_t st, int checkpoint) {
+  int rc;
+  const DslashArgs a = norm_args(w);
+  rc = check_launch(w->ctx, launch_dslash(w->prec, w->recon, w->cfg_norm.nr, MODE_NORM,
+                                          w->prec, a, w->cfg_norm.block, st));
+  if (rc) return rc;
+  if ((rc = check_launch(w->ctx, launch_cg_finish(0, vec_args(w, 0), st)))) return rc;  // alpha
+  const DslashArgs b = update_args(w);
   rc = check_launch(w->ctx, launch_dslash(w->prec, w->recon, w->cfg_update.nr, MODE_UPDATE,
                                           w->prec, b, w->cfg_update.block, st));
   if (rc) return rc;
@@ -313,6 +328,30 @@ int cg_run(CGWork *w, int block_iters, bool graph, cudaStream_t st) {
   return SQ_OK;
 }
 
+// The same by the resident kernel: each round runs iterations until the system
+// wants an FP64 residual, and the pair that computes it; four rounds (empty
+// once the system is done) between two looks at the state.
+int cg_run_resident(CGWork *w, cudaStream_t st) {
+  int rc;
+  const DslashArgs a = norm_args(w), b = update_args(w);
+  int *fault = static_cast<int *>(w->resident);
+  int h_fault = 0;
+  do {
+    for (int k = 0; k < 4; ++k) {
+      if ((rc = cg_enqueue_resident(w, a, b, st))) return rc;
+      if ((rc = cg_enqueue_ru(w, st))) return rc;
+    }
+    SQ_CUDA_TRY(cudaMemcpyAsync(&h_fault, fault, sizeof(int), cudaMemcpyDeviceToHost, st));
+    if ((rc = cg_slots_download(w, st))) return rc;
+    SQ_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h_fault) {
+      SQ_CUDA_TRY(cudaMemsetAsync(fault, 0, sizeof(int), st));
+      return SQ_ERR_TIMEOUT;
+    }
+  } while (any_running(w));
+  return SQ_OK;
+}
+
 int slot_status_to_sq(int s) {
   switch (s) {
     case SLOT_CONVERGED: return SQ_OK;
@@ -327,6 +366,11 @@ int slot_status_to_sq(int s) {
 
 void fill_launch_stats(const CGWork *w, sq_cg_stats *st) {
   if (!st) return;
+  if (w->resident_block) {
+    st->oe_block = st->eo_block = w->resident_block;
+    st->oe_rhs_tile = st->eo_rhs_tile = 1;
+    return;
+  }
   st->oe_block = std::min(w->cfg_norm.block, dslash_max_block(w->prec, w->cfg_norm.nr));
   st->oe_rhs_tile = w->cfg_norm.nr;
   st->eo_block = std::min(w->cfg_update.block, dslash_max_block(w->prec, w->cfg_update.nr));

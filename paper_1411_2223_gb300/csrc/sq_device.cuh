@@ -214,15 +214,24 @@ __device__ __forceinline__ uint32_t encode_word(float re, float im, float inv) {
 //   F64: double2 plane per colour; F32: float4 (c0, c1) + float2 (c2) planes;
 //   I16: one uint4 per site = 3 code words + FP32 norm.
 
+// CO: loads of fields that change while the kernel runs (the resident CG), by
+// coherent instructions; otherwise through the read-only path.
+template <bool CO, typename T>
+__device__ __forceinline__ T ld_field(const T *p) {
+  if constexpr (CO) return *p;
+  else return __ldg(p);
+}
+
 template <int PREC> struct SpinorIO;
 
 template <> struct SpinorIO<PREC_F64> {
   using R = double;
+  template <bool CO = false>
   static __device__ __forceinline__ Vec3<double> load(const char *base, int S, int i) {
     const double2 *p = reinterpret_cast<const double2 *>(base);
     Vec3<double> v;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) v.c[c] = __ldg(p + (size_t)c * S + i);
+    for (int c = 0; c < 3; ++c) v.c[c] = ld_field<CO>(p + (size_t)c * S + i);
     return v;
   }
   static __device__ __forceinline__ void store(char *base, int S, int i, const Vec3<double> &v) {
@@ -234,9 +243,10 @@ template <> struct SpinorIO<PREC_F64> {
 
 template <> struct SpinorIO<PREC_F32> {
   using R = float;
+  template <bool CO = false>
   static __device__ __forceinline__ Vec3<float> load(const char *base, int S, int i) {
-    float4 a = __ldg(reinterpret_cast<const float4 *>(base) + i);
-    float2 b = __ldg(reinterpret_cast<const float2 *>(base + (size_t)16 * S) + i);
+    float4 a = ld_field<CO>(reinterpret_cast<const float4 *>(base) + i);
+    float2 b = ld_field<CO>(reinterpret_cast<const float2 *>(base + (size_t)16 * S) + i);
     Vec3<float> v;
     v.c[0] = make_float2(a.x, a.y);
     v.c[1] = make_float2(a.z, a.w);
@@ -252,8 +262,9 @@ template <> struct SpinorIO<PREC_F32> {
 template <> struct SpinorIO<PREC_I16> {
   using R = float;
   // values in code units together with the dequantisation factor n/32767
+  template <bool CO = false>
   static __device__ __forceinline__ Vec3<float> load_codes(const char *base, int i, float &scale) {
-    uint4 w = __ldg(reinterpret_cast<const uint4 *>(base) + i);
+    uint4 w = ld_field<CO>(reinterpret_cast<const uint4 *>(base) + i);
     Vec3<float> v;
     v.c[0] = decode_word(w.x);
     v.c[1] = decode_word(w.y);
@@ -261,9 +272,10 @@ template <> struct SpinorIO<PREC_I16> {
     scale = __uint_as_float(w.w) * (1.f / 32767.f);
     return v;
   }
+  template <bool CO = false>
   static __device__ __forceinline__ Vec3<float> load(const char *base, int S, int i) {
     float s;
-    Vec3<float> v = load_codes(base, i, s);
+    Vec3<float> v = load_codes<CO>(base, i, s);
 #pragma unroll
     for (int c = 0; c < 3; ++c) { v.c[c].x *= s; v.c[c].y *= s; }
     return v;

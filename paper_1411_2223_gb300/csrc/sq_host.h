@@ -97,6 +97,8 @@ struct DslashConfig {
 
 DslashConfig tuned_dslash(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs,
                           int mode, cudaStream_t st);
+// Is the shape given by the file SQ_TUNE_CACHE named?
+bool tuned_pinned(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs, int mode);
 Tuner *tuner_create();
 void tuner_destroy(Tuner *);
 
@@ -120,6 +122,8 @@ struct CGWork {
   int exec_iters = 0;
   int exec_kernels = 0;       // kernels per replay
   DslashConfig cfg_norm, cfg_update, cfg_ru_plain, cfg_ru_resid;
+  void *resident = nullptr;   // cg_resident.cu: fault flag, barrier, second p
+  int resident_block = 0;     // threads per block of the resident kernel; 0: launched kernels
 
   ~CGWork();
 };
@@ -130,7 +134,7 @@ void cg_slot_setup(CGWork *w, int slot, double mass, double tol, double delta, i
 int cg_slots_upload(CGWork *w, cudaStream_t st);
 int cg_slots_download(CGWork *w, cudaStream_t st);
 // Launch sequences.
-int cg_enqueue_init(CGWork *w, int guess, cudaStream_t st);
+int cg_enqueue_init(CGWork *w, int guess, cudaStream_t st, bool xpay = true);
 int cg_enqueue_ru(CGWork *w, cudaStream_t st);
 int cg_enqueue_xpay(CGWork *w, cudaStream_t st);
 // Reliable updates may follow every RU_PERIOD-th iteration (a checkpoint).
@@ -140,6 +144,15 @@ int cg_enqueue_iteration(CGWork *w, cudaStream_t st, int checkpoint);
 int cg_enqueue_block(CGWork *w, int k, bool graph, cudaStream_t st);
 // Run until no slot is running; host polls the slot state after each block.
 int cg_run(CGWork *w, int block_iters, bool graph, cudaStream_t st);
+int cg_run_resident(CGWork *w, cudaStream_t st);
+// The one-system CG as a resident kernel (cg_resident.cu): iterations of one
+// launch (a few ms at most, so that other streams' kernels get in between),
+// and its block for a workspace it is the faster form for (else 0).
+constexpr int RESIDENT_STEPS = 128;
+size_t cg_resident_bytes(const sq_ctx *ctx, size_t fb);
+int cg_resident_block(const CGWork *w);
+int cg_enqueue_resident(CGWork *w, const DslashArgs &norm, const DslashArgs &update,
+                        cudaStream_t st);
 int slot_status_to_sq(int slot_status);
 inline bool cg_slot_live(int s) { return s == SLOT_RUNNING || s == SLOT_WAIT || s == SLOT_INIT; }
 void drop_multishift_works(const sq_ctx *ctx, int gauge_id);  // gauge_id < 0: all

@@ -11,6 +11,7 @@
 #include <fstream>
 #include <map>
 #include <mutex>
+#include <set>
 #include <sstream>
 #include <string>
 #include <utility>
@@ -23,6 +24,7 @@ namespace sq {
 struct Tuner {
   std::mutex mu;
   std::map<std::string, DslashConfig> cache;
+  std::set<std::string> pinned;  // keys read from the file
   std::string path;
 };
 
@@ -41,12 +43,22 @@ Tuner *tuner_create() {
     std::ifstream in(t->path);
     std::string key;
     DslashConfig c;
-    while (in >> key >> c.block >> c.nr) t->cache[key] = c;
+    while (in >> key >> c.block >> c.nr) {
+      t->cache[key] = c;
+      t->pinned.insert(key);
+    }
   }
   return t;
 }
 
 void tuner_destroy(Tuner *t) { delete t; }
+
+bool tuned_pinned(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs, int mode) {
+  Tuner *t = ctx->tuner;
+  if (!t) return false;
+  std::lock_guard<std::mutex> lk(t->mu);
+  return t->pinned.count(tune_key(gf.g, prec, recon, nrhs, mode)) != 0;
+}
 
 static void tuner_save(Tuner *t) {
   if (t->path.empty()) return;
