@@ -28,9 +28,30 @@ void set_last_cuda_error(cudaError_t e, const char *what, const char *file, int 
                 file, line);
 }
 
-LinkScales GaugeField::scales(int prec, int recon) const {
+// Share of a field's links (both parities, `total` bytes in the form in use)
+// that the one-system kernels leave in L2 (evict-normal) for the next
+// iteration; the rest is marked evict-first.  The whole of what fits beside
+// the vectors, a part of what does not, and nothing of fields so large that the
+// part saves less than the vectors' evictions cost.  us per CG iteration with
+// all links evict-first and with the rule (sweep of 0 to 128 MB, one box):
+//   MB of links   47    82    125   150   188   207   245   294   442
+//   FP32          19.4  26.2  32.2  34.9  65.0  54.9  65.9  68.6  88.8  (188: FP64)
+//                 16.4  20.9  27.3  28.7  63.2  51.5  63.2  65.2  88.8
+// At 442 MB 48 MB cost 0.4 us, at 590 MB (20^3 x 64) 40 MB cost 5 of 114 us.
+static float l2_share(double total) {
+  const double mb = total * 1e-6;
+  const double kept = mb <= 88 ? mb : mb <= 200 ? 52 : mb <= 320 ? 36 : 0;
+  return mb > 0 ? (float)(kept / mb) : 0.f;
+}
+
+LinkScales GaugeField::scales(int prec, int recon, int nrhs) const {
   LinkScales s;
   s.keep = 0;
+  s.share = 0.f;
+  if (nrhs == 1) {
+    const double total = 2.0 * (double)link_site_bytes(prec, prec == PREC_F64 ? 18 : recon) * g.stride;
+    s.share = l2_share(total);
+  }
   s.fat_k = fat_scale / 32767.f;
   s.long_k = long_scale / 32767.f;
   s.recon_d = (long_s != 0) ? 1.0 / long_s : 0.0;
@@ -419,7 +440,7 @@ extern "C" int dslash_apply(sq_ctx *ctx, int gauge_id, int out_parity, int prec,
   a.g = gf->g;
   a.out_parity = out_parity;
   a.links = gf->link_ptr(prec, long_recon, out_parity);
-  a.ls = gf->scales(prec, long_recon);
+  a.ls = gf->scales(prec, long_recon, 1);
   a.in = static_cast<const char *>(in_dev);
   a.out = static_cast<char *>(out_dev);
   a.nrhs = 1;
@@ -498,7 +519,7 @@ extern "C" int mdagm_apply(sq_ctx *ctx, int gauge_id, int prec, int long_recon, 
   a.g = gf->g;
   a.nrhs = 1;
   a.gate = GATE_NONE;
-  a.ls = gf->scales(prec, long_recon);
+  a.ls = gf->scales(prec, long_recon, 1);
   a.out_parity = 1;
   a.links = gf->link_ptr(prec, long_recon, 1);
   a.in = static_cast<const char *>(in_dev);

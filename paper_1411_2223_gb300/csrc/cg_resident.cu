@@ -97,7 +97,7 @@ template <int PREC, int RECON> struct DirLinks {
 template <int RECON> struct DirLinks<PREC_I16, RECON> {
   I16Words<RECON> w;
   __device__ __forceinline__ void load(const DslashArgs &a, int i, int mu) {
-    i16_load_words<RECON>(a.links, a.g.stride, i, mu, w, false);
+    i16_load_words<RECON>(a.links, a.g.stride, i, mu, w, a.ls);
   }
 };
 template <int RECON> struct DirLinks<PREC_F64, RECON> {

@@ -166,11 +166,11 @@ __device__ __forceinline__ void put4(uint32_t *w, uint4 q) {
 
 template <int RECON>
 __device__ __forceinline__ void i16_load_words(const char *links, int S, int i, int mu,
-                                               I16Words<RECON> &d, bool keep) {
+                                               I16Words<RECON> &d, const LinkScales &ls) {
   using LL = LinkLayout<PREC_I16, RECON>;
   const char *fat = links + (size_t)mu * LL::mu_bytes * S;
   const char *lng = fat + (size_t)LL::fat_bytes * S;
-  const uint64_t pol = l2_link_policy(keep);
+  const uint64_t pol = l2_link_policy(ls.keep, ls.share);
 #pragma unroll
   for (int k = 0; k < 4; ++k) put4(d.w + 4 * k, ld_stream_u4(fat + ((size_t)k * S + i) * 16, pol));
   {
@@ -274,7 +274,7 @@ __device__ __forceinline__ void i16_hops(const DslashArgs &a, const LinkScales &
                                          I16Words<RECON> &buf) {
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
-    if (mu > 0) i16_load_words<RECON>(a.links, a.g.stride, i, mu, buf, ls.keep);
+    if (mu > 0) i16_load_words<RECON>(a.links, a.g.stride, i, mu, buf, ls);
     i16_dir<RECON, NR, false>(a, ls, sc, mu, buf.w, r0, active, acc);
   }
 }
@@ -427,7 +427,7 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
   constexpr bool XS = IN == IN_XS;
   const Geom &g = a.g;
   const int S = g.stride;
-  const uint64_t pol = l2_link_policy(ls.keep);
+  const uint64_t pol = l2_link_policy(ls.keep, ls.share);
   FxAcc s[NR];
   bool odd[NR];  // a neighbour outside the fixed-point range
 #pragma unroll
@@ -770,7 +770,7 @@ __device__ __forceinline__ void multi_hops(const DslashArgs &a, const LinkScales
                                            float4 *stage, Vec3<float> (&vf)[2][NR]) {
   const Geom &g = a.g;
   const int S = g.stride;
-  const uint64_t pol = l2_link_policy(ls.keep);
+  const uint64_t pol = l2_link_policy(ls.keep, ls.share);
   static_assert(NR <= 4, "FP32 tiles hold 1, 2 or 4 systems");
   constexpr bool kEpi = EpiStage<MODE, RECON, NR>::V > 0;
   Vec3<float> vl[2][NR];  // long pair
@@ -824,7 +824,7 @@ template <int RECON> struct FirstLinks<PREC_I16, RECON> {
   static constexpr bool kUsed = true;
   I16Words<RECON> buf;
   __device__ __forceinline__ void load(const DslashArgs &a, const LinkScales &ls, int i) {
-    i16_load_words<RECON>(a.links, a.g.stride, i, 0, buf, ls.keep);
+    i16_load_words<RECON>(a.links, a.g.stride, i, 0, buf, ls);
   }
 };
 
@@ -901,7 +901,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
   extern __shared__ float4 dyn_smem[];
   if constexpr (kStaged) {
     if (i < g.vh) {
-      const uint64_t pol = l2_link_policy(ls.keep);
+      const uint64_t pol = l2_link_policy(ls.keep, ls.share);
       stage_half<RECON, 0>(a.links, S, i, 0, dyn_smem, pol);
       stage_half<RECON, 1>(a.links, S, i, 0, dyn_smem, pol);
     }

@@ -282,7 +282,7 @@ struct FullOps {
     a.g = gf->g;
     a.out_parity = out_parity;
     a.links = gf->link_ptr(prec, 18, out_parity);
-    a.ls = gf->scales(prec, 18);
+    a.ls = gf->scales(prec, 18, 1);
     a.in = in;
     a.out = out;
     a.in_fb = a.out_fb = spinor_bytes(prec, gf->g.stride);

@@ -296,7 +296,7 @@ int ms_enqueue_iteration(MsWork *w, cudaStream_t st) {
   a.gate = GATE_RUNNING;
   a.out_parity = 1;
   a.links = w->gf->link_ptr(w->prec, w->recon, 1);
-  a.ls = w->gf->scales(w->prec, w->recon);
+  a.ls = w->gf->scales(w->prec, w->recon, 1);
   a.in = pb;
   a.out = w->t;
   if (launch_dslash(w->prec, w->recon, 1, MODE_PLAIN, w->prec, a, w->cfg.block, st)) return SQ_ERR_ARG;

@@ -143,7 +143,7 @@ static DslashArgs dslash_args(CGWork *w, int prec, int recon, int out_parity) {
   a.g = w->gf->g;
   a.out_parity = out_parity;
   a.links = w->gf->link_ptr(prec, recon, out_parity);
-  a.ls = w->gf->scales(prec, recon);
+  a.ls = w->gf->scales(prec, recon, w->nrhs);
   a.nrhs = w->nrhs;
   a.slots = w->slots_d;
   return a;

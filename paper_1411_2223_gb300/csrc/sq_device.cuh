@@ -156,8 +156,12 @@ __device__ __forceinline__ void reconstruct_row2(Mat3<R> &m, R f) {
 // keep = true: another tile of the same launch reads these links again soon
 // (its blocks are adjacent in the launch order), so they stay evict-normal;
 // the last reader marks them evict-first.
-__device__ __forceinline__ uint64_t l2_link_policy(bool keep) {
+__device__ __forceinline__ uint64_t l2_link_policy(bool keep, float share) {
   uint64_t p;
+  if (!keep && share > 0.f) {
+    asm("createpolicy.fractional.L2::evict_normal.L2::evict_first.b64 %0, %1;" : "=l"(p) : "f"(share));
+    return p;
+  }
   if (keep) asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   else asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
@@ -357,6 +361,7 @@ struct LinkScales {
   float recon_f;    // 12-real: row2 = recon_f * conj(row0 x row1) in stored units
   double recon_d;   // same, FP64 kernels
   int keep;         // set in the kernel: links read again by a later tile
+  float share;      // of the links' lines, kept in L2 from launch to launch
   int fixed;        // F64, 18-real: the links are fixed-point words (sq_fixed.cuh)
   int fixed_exp;    // ... of value word * 2^(fixed_exp - FX_BITS)
 };
@@ -372,7 +377,7 @@ template <int RECON> struct LinkIO<PREC_F64, RECON> {
                                                    const LinkScales &ls, Mat3<double> m[2]) {
     const char *base = links + (size_t)mu * LL::mu_bytes * S;
     if (KIND == 1) base += (size_t)LL::fat_bytes * S;
-    const uint64_t pol = l2_link_policy(ls.keep);
+    const uint64_t pol = l2_link_policy(ls.keep, ls.share);
     constexpr int ne = (KIND == 0 || RECON == 18) ? 9 : 6;  // stored elements per matrix
 #pragma unroll
     for (int k = 0; k < ne; ++k) {
@@ -388,7 +393,7 @@ template <int RECON> struct LinkIO<PREC_F64, RECON> {
                                               const LinkScales &ls, Mat3<double> m[4]) {
     const char *fat = links + (size_t)mu * LL::mu_bytes * S;
     const char *lng = fat + (size_t)LL::fat_bytes * S;
-    const uint64_t pol = l2_link_policy(ls.keep);
+    const uint64_t pol = l2_link_policy(ls.keep, ls.share);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       m[0].e[k] = ld_stream_d2(fat + ((size_t)k * S + i) * 16, pol);
@@ -423,7 +428,7 @@ template <int RECON> struct LinkIO<PREC_F32, RECON> {
                                                    const LinkScales &ls, Mat3<float> m[2]) {
     const char *base = links + (size_t)mu * LL::mu_bytes * S;
     if (KIND == 1) base += (size_t)LL::fat_bytes * S;
-    const uint64_t pol = l2_link_policy(ls.keep);
+    const uint64_t pol = l2_link_policy(ls.keep, ls.share);
     constexpr int nq = (KIND == 0 || RECON == 18) ? 9 : 6;
     constexpr int ne = (KIND == 0 || RECON == 18) ? 9 : 6;  // stored elements per matrix
     float4 q[nq];
@@ -448,7 +453,7 @@ template <int RECON> struct LinkIO<PREC_F32, RECON> {
                                               const LinkScales &ls, Mat3<float> m[4]) {
     const char *fat = links + (size_t)mu * LL::mu_bytes * S;
     const char *lng = fat + (size_t)LL::fat_bytes * S;
-    const uint64_t pol = l2_link_policy(ls.keep);
+    const uint64_t pol = l2_link_policy(ls.keep, ls.share);
     float4 q[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) q[k] = ld_stream_f4(fat + ((size_t)k * S + i) * 16, pol);
@@ -501,7 +506,7 @@ template <int RECON> struct LinkIO<PREC_I16, RECON> {
                                               const LinkScales &ls, Mat3<float> m[4]) {
     const char *fat = links + (size_t)mu * LL::mu_bytes * S;
     const char *lng = fat + (size_t)LL::fat_bytes * S;
-    const uint64_t pol = l2_link_policy(ls.keep);
+    const uint64_t pol = l2_link_policy(ls.keep, ls.share);
     uint32_t w[18];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {

@@ -61,7 +61,8 @@ struct GaugeField {
     if (prec == PREC_F64 && f64_12_fixed) recon = 18;
     return static_cast<const char *>(links[prec][recon == 12][parity]);
   }
-  LinkScales scales(int prec, int recon) const;
+  // nrhs 1: for operators on one vector, which may keep a share of the links in L2
+  LinkScales scales(int prec, int recon, int nrhs = 0) const;
 };
 
 struct sq_ctx_impl;
