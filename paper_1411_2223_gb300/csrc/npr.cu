@@ -27,17 +27,26 @@
 //   4. per operator and output, the 256-term sum over (A, C) of
 //      +-P[A][C ^ t2][a1][a4] Q[C][A ^ t1][a3][a2], t = S ^ F.
 // The arithmetic (about 1.6 MFLOP per hypercube for 8 operators, against
-// 14 KB of input) runs on the integer multiply-add units in the two-word
-// fixed-point form of sq_fixed.cuh, 54 bits relative to block scales: one per
-// hypercube for the links, for each flavour's propagators, for P and for Q
-// (npr_kernel).  A hypercube whose inputs or averaged links do not fit that
-// form (infinities, NaN, elements near the ends of FP64, links far from
-// unitary) is marked there and computed by npr_fp64_kernel in FP64.
+// 14 KB of input) is FP64 in its results but not in its units, which GB300
+// has few of (npr_kernel):
+//   - steps 2 and 3 run on the integer multiply-add units in the two-word
+//     fixed-point form of sq_fixed.cuh, 54 to 57 bits relative to block
+//     scales: one per hypercube for the links and for each flavour's
+//     propagators;
+//   - step 4, four fifths of the work, on the tensor cores: P and Q, at one
+//     scale each, are cut into six signed 9-bit digits, which FP16 holds
+//     exactly, and the digits' products are summed over the 256 (A, C) by
+//     mma.sync with FP32 accumulators, exactly (256 256 256 = 2^24).
+// A hypercube whose inputs or averaged links do not fit that form (infinities,
+// NaN, elements near the ends of FP64, links far from unitary) is marked there
+// and computed by npr_fp64_kernel in FP64.
 // Per-hypercube results are written when asked for; the sums over hypercubes
 // go through per-CTA partials and a fixed-order second pass, so they do not
 // depend on scheduling.
 #include <cmath>
 #include <cstdint>
+
+#include <cuda_fp16.h>
 
 #include "sq_fixed.cuh"
 #include "sq_host.h"
@@ -68,7 +77,7 @@ int spin_taste_sign(int s, int f, int a) {
 }
 
 constexpr int kThreads = 512;    // npr_fp64_kernel
-constexpr int kFxThreads = 288;  // npr_kernel
+constexpr int kFxThreads = 512;  // npr_kernel
 constexpr int kMaxOps = SQ_NPR_MAX_OPS;
 constexpr int kItemsPerThread = (kMaxOps * 81 + kThreads - 1) / kThreads;
 constexpr int kTri = 136;                  // corner pairs A <= D
@@ -319,24 +328,29 @@ __global__ void __launch_bounds__(kThreads, 1) npr_fp64_kernel(const NprArgs a) 
 // ------------------------------------------------------ fixed-point kernel
 // Elements in shared memory are int4 (re.l, re.h, im.l, im.h) with balanced
 // low words of 27 bits.  Bits at a block's scale: 55 for the propagators, 56
-// for the links and their averages, 54 (53 with 2 slices) and 55 for P and Q,
-// whose products are added 512 at a time: over a thread's slice
-//   |hi| <= (512 / slices) 2^27 2^28 < 2^63,
-//   |mid| <= (512 / slices) (2^27 2^26 + 2^26 2^28) < 2^63.
-// The dropped products of two low words are below 2^-57 of the blocks' scales.
+// for the links and their averages.
 //
-// The contraction takes most of the time.  A thread owns the outputs (a4, a2)
-// of one (operator, a1, a3), 9 complex sums, over one slice of A: two groups
-// of 3 elements are loaded for 9 complex terms of 12 multiply-adds each, so
-// the shared-memory reads stay below the multiply-add time.  The slices (2 to
-// 16, as many as fill 288 threads for the number of operators) are added by
-// shuffles; integer sums do not depend on the order.  Two CTAs of 9 warps per
-// SM (96 registers, a few spilled) and one of 164 registers measured the same.
+// Contraction.  With i, j = 0 .. 5 the digits of P and Q from the top,
+//   P = sum_i p_i 512^(5-i), |p_i| <= 256,
+// row 18 i + 2 (3 a1 + a4) + (0 re, 1 im) of the [108] x [256] matrix of p
+// digits and column 18 j + 2 (3 a3 + a2) + (0, 1) of the [256] x [108] matrix
+// of q digits give C = one 108 x 108 product per operator, of which the blocks
+// i + j <= 6 are needed (the others are below 2^-59 of the scales' product):
+// 75 of the 7 x 14 tiles of m16n8k16, 16 steps of k each.  The matrices lie in
+// shared memory by rows of k = (A, D) and (B, C) -- 240 bytes, so that the
+// eight rows an ldmatrix reads fall on different banks -- and an operator's
+// permutation D = C ^ t2, B = A ^ t1 is in the rows' addresses, its signs in an
+// XOR of the fragments.  The sums of digit pairs of one i + j are added as
+// integers, the seven of them to two 64-bit words, and these converted once.
 //
 // 8 operators at 20^3 x 64: 37.2 ms with FP64 FMAs (their pipe 93 % busy),
-// 15.6 ms here, the multiply-add pipe 61 % busy (mad.wide.s32 issues 32 lanes
-// per clock and SM).  Error of a hypercube against long double 2.0e-16 to
-// 2.3e-16, with FP64 FMAs (three per complex term) 4.6e-16.
+// 15.2 ms with the contraction on the integer units too (three mad.wide.s32
+// per real product, 32 lanes a clock and SM: 62 of its 147 thousand cycles per
+// hypercube at best), 9.8 ms here: about 40 thousand cycles up to the digits
+// and 7 thousand per operator, of which the tensor cores (938 multiply-adds a
+// clock and SM for mma.sync) take 2.6 and the ldmatrix reads 3.7.  Error of a
+// hypercube against long double 3.2e-16 to 3.6e-16, with FP64 FMAs (three per
+// complex term) 4.6e-16.
 struct FxC { Fx re, im; };
 struct Wide { long long hr, mr, hi, mi; };
 
@@ -382,13 +396,15 @@ __device__ __forceinline__ FxC fx_u(const int4 *ut, int x, int y, int i, int j) 
   return u;
 }
 
-constexpr int kFxRow = 16 * 9 + 2;      // padded row of P: slices of A fall on different banks
-constexpr int kFxP = 16 * kFxRow, kFxQ = 256 * 9;
-constexpr size_t kFxSmem = sizeof(int4) * (kTri * 9 + 4 * 16 * 9 + kFxP + kFxQ);
 constexpr long long kFxMost = 1ll << (FX_LOW + 30);  // two words hold values below this
 constexpr int kPropBits = FX_BITS, kLinkBits = 56;   // bits at the blocks' scales
 constexpr int kMidBits = 55;                         // ... of U G4 and U G2
-template <int SLICES> struct PQBits { static constexpr int p = SLICES >= 4 ? 54 : 53, q = 55; };
+constexpr int kDigits = 6, kDigitBits = 9;
+constexpr int kPQBits = kDigits * kDigitBits - 1;    // P and Q: |v| <= 2^53
+constexpr int kRowHalfs = 120;                       // a row of digits: 108, padded to 240 bytes
+constexpr size_t kDigitBytes = (size_t)256 * kRowHalfs * 2;
+constexpr int kFxUG = kTri * 9 + 4 * 16 * 9;  // int4 of the links and propagators
+constexpr size_t kFxSmem = sizeof(int4) * (kFxUG + 2 * 2304) + 2 * kDigitBytes;
 
 struct FxShared {
   int e[5];                    // largest biased exponents: 4 flavours, links
@@ -404,79 +420,171 @@ __device__ __forceinline__ long long fx_scaled(double v, int biased_top) {
   return ((long long)a.h << FX_LOW) + a.l;
 }
 
-template <int SLICES>
-__device__ __forceinline__ void fx_contract(const int4 *ps, const int4 *qs, NprOp op, int a1, int a3,
-                                            int slice, Wide (&w)[9]) {
-#pragma unroll 1
-  for (int A = slice; A < 16; A += SLICES) {
-    const int4 *pa = ps + A * kFxRow + 3 * a1;
-    const int4 *qa = qs + (A ^ op.t1) * 9 + 3 * a3;
-    const unsigned sa = ((op.neg1 >> A) & 1) ? 0xffffu : 0u;
-    const unsigned neg = op.neg2 ^ sa;
-#pragma unroll 1
-    for (int C = 0; C < 16; ++C) {
-      const int s = -(int)((neg >> C) & 1);
-      FxC p[3], q[3];
+// C is kept for the needed blocks only, by rows of digit i: columns 0 ..
+// 18 (7 - i) - 1 (at most 108).
+__device__ __forceinline__ int c_width(int i) { return i == 0 ? 108 : 18 * (7 - i); }
+__device__ __forceinline__ int c_base(int i) {  // of row 18 i
+  return 18 * (i == 0 ? 0 : 108 + 18 * ((i - 1) * 7 - (i * (i - 1)) / 2));
+}
+
+constexpr int kCFloats = 18 * (108 + 108 + 90 + 72 + 54 + 36);
+static_assert(2 * kCFloats * sizeof(float) <= 2 * 2304 * sizeof(longlong2), "two C fit where P and Q were");
+
+__device__ __forceinline__ void ldsm4t(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// A warp's tiles of C: m-tile, first n-tile and number of n-tiles (at most 6).
+// Needed n-tiles of the seven m-tiles: 14, 14, 14, 12, 9, 7, 5.
+__device__ __forceinline__ void warp_tiles(int warp, int &mt, int &nt, int &n) {
+  // mt (4 bits), nt (4), n (4) of the 16 warps
+  constexpr unsigned short t[16] = {0x005, 0x055, 0x0a4, 0x105, 0x155, 0x1a4, 0x205, 0x255,
+                                    0x2a4, 0x306, 0x366, 0x405, 0x454, 0x504, 0x543, 0x605};
+  unsigned v = 0;
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        p[k] = fx_load(pa + (C ^ op.t2) * 9 + k);
-        q[k] = fx_load(qa + C * 144 + k);
-        q[k].re = fx_flip(q[k].re, s);
-        q[k].im = fx_flip(q[k].im, s);
-      }
+  for (int k = 0; k < 16; ++k)
+    if (k == warp) v = t[k];
+  mt = v >> 8;
+  nt = (v >> 4) & 15;
+  n = v & 15;
+}
+
+// The digit products of one operator into c (see above) for N n-tiles.
+template <int N>
+__device__ __forceinline__ void digit_tiles(unsigned pd, unsigned qd, NprOp op, float *c, int mt, int nt) {
+  const int lane = threadIdx.x & 31;
+  float acc[N][4];
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
+  for (int u = 0; u < N; ++u)
 #pragma unroll
-        for (int m = 0; m < 3; ++m) wide_mac(w[3 * k + m], p[k], q[m]);
+    for (int e = 0; e < 4; ++e) acc[u][e] = 0.f;
+  // the row this lane addresses: matrices (k 0-7, m 0-7), (k 0-7, m 8-15),
+  // (k 8-15, m 0-7), (k 8-15, m 8-15) of A; (k 0-7, n 0-7), (k 8-15, n 0-7),
+  // (k 0-7, n 8-15), (k 8-15, n 8-15) of B
+  const int ka = (lane & 7) + ((lane >> 4) & 1) * 8, kb = (lane & 7) + ((lane >> 3) & 1) * 8;
+  const unsigned a0 = pd + (unsigned)((ka ^ op.t2) * kRowHalfs + mt * 16 + ((lane >> 3) & 1) * 8) * 2;
+  const unsigned b0 = qd + (unsigned)(kb * kRowHalfs + nt * 8 + ((lane >> 4) & 1) * 8) * 2;
+  // signs of the k this lane's fragment registers hold: 2t, 2t + 1 and 8 more
+  const int t2 = 2 * (lane & 3);
+  auto mask = [&](int k) {
+    return (((op.neg2 >> k) & 1u) << 15) | (((op.neg2 >> (k + 1)) & 1u) << 31);
+  };
+  const unsigned lo = mask(t2), hi = mask(t2 + 8);
+#pragma unroll 4
+  for (int A = 0; A < 16; ++A) {
+    const unsigned sa = ((op.neg1 >> A) & 1) ? 0x80008000u : 0u;
+    unsigned a[4], b[(N + 1) / 2][4];
+    ldsm4t(a, a0 + (unsigned)(A * 16 * kRowHalfs * 2));
+    const unsigned ba = b0 + (unsigned)((A ^ op.t1) * 16 * kRowHalfs * 2);
+#pragma unroll
+    for (int u = 0; u < (N + 1) / 2; ++u) ldsm4t(b[u], ba + u * 32);
+    a[0] ^= lo ^ sa;
+    a[1] ^= lo ^ sa;
+    a[2] ^= hi ^ sa;
+    a[3] ^= hi ^ sa;
+#pragma unroll
+    for (int u = 0; u < N; ++u) mma16816(acc[u], a, b[u / 2][2 * (u & 1)], b[u / 2][2 * (u & 1) + 1]);
+  }
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    const int row = mt * 16 + (lane >> 2) + v * 8, i = row / 18, w = c_width(i);
+    float *cr = c + c_base(i) + (row - 18 * i) * w;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      const int col = (nt + u) * 8 + t2;  // even, as every width is
+      if (row < 108 && col < w) *reinterpret_cast<float2 *>(cr + col) = make_float2(acc[u][2 * v], acc[u][2 * v + 1]);
     }
   }
 }
 
-template <int SLICES>
-__global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constant__ NprArgs a) {
+// ... by the 16 warps.
+__device__ __forceinline__ void digit_products(unsigned pd, unsigned qd, NprOp op, float *c, int mt, int nt,
+                                               int n) {
+  switch (n) {
+    case 3: digit_tiles<3>(pd, qd, op, c, mt, nt); break;
+    case 4: digit_tiles<4>(pd, qd, op, c, mt, nt); break;
+    case 5: digit_tiles<5>(pd, qd, op, c, mt, nt); break;
+    default: digit_tiles<6>(pd, qd, op, c, mt, nt);
+  }
+}
+
+// Sums over (A, C) of p q for the real parts (ra, rb) of output elements
+// pe, qe: hi + lo 2^-27 in units of 512^7.
+__device__ __forceinline__ void digit_sum(const float *c, int ra, int rb, long long &hi, long long &lo) {
+  int level[7];
+#pragma unroll
+  for (int s = 0; s < 7; ++s) level[s] = 0;
+#pragma unroll
+  for (int i = 0; i < kDigits; ++i)
+#pragma unroll
+    for (int j = 0; j < kDigits; ++j)
+      if (i + j <= 6)
+        level[i + j] += __float2int_rn(c[c_base(i) + ra * c_width(i) + 18 * j + rb]);
+  hi = ((((long long)level[0] * 512 + level[1]) * 512 + level[2]) * 512) + level[3];
+  lo = (((long long)level[4] * 512 + level[5]) * 512) + level[6];
+}
+
+__global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constant__ NprArgs a) {
   extern __shared__ int4 fsm[];
   __shared__ FxShared sh;
-  int4 *ut = fsm;              // [pair A <= D][3][3]
-  int4 *gs = ut + kTri * 9;    // [flavour][corner][3][3]
-  int4 *ps = gs + 4 * 16 * 9;  // [A][D][a1][a4], rows of kFxRow
-  int4 *qs = ps + kFxP;        // [C][B][a3][a2]
+  int4 *ut = fsm;                       // [pair A <= D][3][3]
+  int4 *gs = ut + kTri * 9;             // [flavour][corner][3][3]
+  longlong2 *pq = reinterpret_cast<longlong2 *>(gs + 4 * 16 * 9);  // P [A][D][9], Q [B][C][9]
+  float *cm = reinterpret_cast<float *>(pq);                       // C, once these are cut
+  __half *pd = reinterpret_cast<__half *>(pq + 2 * 2304);          // digits of P, then of Q
+  const unsigned pd_s = (unsigned)__cvta_generic_to_shared(pd), qd_s = pd_s + (unsigned)kDigitBytes;
   const int tid = threadIdx.x;
-  const int slice = tid % SLICES, tile = (tid / SLICES) % 9, iop = tid / (9 * SLICES);
-  const bool mine = iop < a.nops;
-  const NprOp op = a.ops[mine ? iop : 0];
-  const int a1 = tile / 3, a3 = tile % 3;
-  constexpr int kOwn = (9 + SLICES - 1) / SLICES;  // outputs a thread finishes
-  double2 tot[kOwn];
-#pragma unroll
-  for (int r = 0; r < kOwn; ++r) tot[r] = make_double2(0.0, 0.0);
   if (tid == 0) {
     for (int k = 0; k < 5; ++k) sh.e[k] = 0;
     sh.bad = 0;
     sh.most[0] = sh.most[1] = 0;
   }
+  // columns 108 .. 119 of the digits meet no needed block, but are multiplied
+  for (int i = tid; i < 2 * 256 * (kRowHalfs - 108); i += kFxThreads)
+    pd[(i / (kRowHalfs - 108)) * kRowHalfs + 108 + i % (kRowHalfs - 108)] = __half(0.f);
+  // this thread's part of an operator's outputs: output o = tid / 4, and the
+  // real (0) or imaginary (1) parts of P and Q
+  const int o = tid >> 2, part = tid & 3;
+  const bool mine = o < 81;
+  const int oe = mine ? o : 0;
+  const int ra = 2 * (3 * (oe / 27) + oe % 3) + (part >> 1);            // P[a1][a4]
+  const int rb = 2 * (3 * ((oe / 3) % 3) + (oe / 9) % 3) + (part & 1);  // Q[a3][a2]
+  int mt, nt, ntiles;
+  warp_tiles(tid >> 5, mt, nt, ntiles);
+  double *sum = reinterpret_cast<double *>(a.partial + (long)blockIdx.x * a.nops * 81);
+  if (mine && part < 2)
+    for (int op = 0; op < a.nops; ++op) sum[2 * (op * 81 + o) + part] = 0.0;
   int h = blockIdx.x;
   if (h < a.nhc)
     issue_loads<kFxThreads>(a, h, reinterpret_cast<double2 *>(gs), reinterpret_cast<double2 *>(ut));
   for (; h < a.nhc; h += gridDim.x) {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    // block scales of the inputs: 864 elements, 3 per thread, 2 of the
-    // propagators' and 1 of the links' (a warp's 32 span two flavours at most)
-    int4 *own[3];
-    double2 raw[3];
+    // block scales of the inputs: 576 elements of the propagators, then 288 of
+    // the links (a warp's 32 span two blocks at most)
+    int4 *own[2];
+    double2 raw[2];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 2; ++k) {
       const int i = tid + k * kFxThreads;
-      if (k < 2) {
+      if (i < 576) {
         own[k] = gs + i;
       } else {
-        const int j = tid, mu = j / 72, m = (j / 9) % 8, e = j % 9;
+        const int j = min(i - 576, 287), mu = j / 72, m = (j / 9) % 8, e = j % 9;
         const int c = ((m >> mu) << (mu + 1)) | (m & ((1 << mu) - 1));
         own[k] = ut + tri(c, c | (1 << mu)) * 9 + e;
       }
       raw[k] = *reinterpret_cast<const double2 *>(own[k]);
       const int b = max(fx_biased(raw[k].x), fx_biased(raw[k].y));
-      const int f = k < 2 ? i / 144 : 4;
+      const int f = min(i / 144, 4);
       const int f0 = __shfl_sync(0xffffffffu, f, 0), f1 = __shfl_sync(0xffffffffu, f, 31);
       const int b0 = __reduce_max_sync(0xffffffffu, f == f0 ? b : 0);
       const int b1 = __reduce_max_sync(0xffffffffu, f == f1 ? b : 0);
@@ -495,10 +603,14 @@ __global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constan
       else fits &= k == 4 ? (e[k] >= 1022 - 1 && e[k] <= 1022 + 2) : (e[k] >= 1022 - 200 && e[k] <= 1022 + 200);
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 2; ++k) {
       const int i = tid + k * kFxThreads;
-      const int top = k < 2 ? e[i / 144] : e[4];
-      const int up = k < 2 ? 0 : kLinkBits - FX_BITS;
+      if (i >= 864) break;
+      int top = e[4];
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        if (i / 144 == f) top = e[f];
+      const int up = i < 576 ? 0 : kLinkBits - FX_BITS;
       *own[k] = fx_word(fx_scaled(raw[k].x, top) << up, fx_scaled(raw[k].y, top) << up);
       if (fx_biased(raw[k].x) == 0) fits &= raw[k].x == 0.0;  // no denormals
       if (fx_biased(raw[k].y) == 0) fits &= raw[k].y == 0.0;
@@ -514,8 +626,8 @@ __global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constan
 #pragma unroll 1
     for (int n = 2; n <= 4; ++n) {  // distance n: U_AD for the 8 C(4, n) pairs A < D
       const int npairs = n == 2 ? 48 : (n == 3 ? 32 : 8);
-      for (int it = tid; it < npairs * 9; it += kFxThreads) {
-        const int k = it / 9, el = it % 9, i = el / 3, j = el % 3;
+      if (tid < npairs * 9) {
+        const int k = tid / 9, el = tid % 9, i = el / 3, j = el % 3;
         int x = 0;  // the (k/8)-th difference mask with n bits
         for (int m = 1, seen = 0; m < 16; ++m)
           if (__popc(m) == n && seen++ == (k >> 3)) {
@@ -559,7 +671,8 @@ __global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constan
       const int which = it >= 768;
       const int rem = it - which * 768;
       const int pair = rem / 3, col = rem % 3;
-      const int x = pair >> 4, y = pair & 15;
+      // P[A][D] in rows (A, D); Q[C][B] in rows (B, C)
+      const int x = which ? pair & 15 : pair >> 4, y = which ? pair >> 4 : pair & 15;
       const int4 *gl = gs + ((which ? 2 : 0) * 16 + x) * 9;
       const int4 *gr = gs + ((which ? 1 : 3) * 16 + y) * 9;
       FxC hcol[3];
@@ -575,7 +688,7 @@ __global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constan
         big |= max(abs64(re), abs64(im)) >= kFxMost;
         hcol[c] = {fx_split(re), fx_split(im)};
       }
-      longlong2 *dst = reinterpret_cast<longlong2 *>(which ? qs + pair * 9 : ps + x * kFxRow + y * 9) + col;
+      longlong2 *dst = pq + which * 2304 + pair * 9 + col;
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
         Wide w = {0, 0, 0, 0};
@@ -604,8 +717,7 @@ __global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constan
     // P and Q at their own scales
     int sc[2];
 #pragma unroll
-    for (int k = 0; k < 2; ++k)
-      sc[k] = max(0, 64 - __clzll((long long)sh.most[k]) - (k ? PQBits<SLICES>::q : PQBits<SLICES>::p));
+    for (int k = 0; k < 2; ++k) sc[k] = max(0, 64 - __clzll((long long)sh.most[k]) - kPQBits);
     __syncthreads();
     if (tid == 0) {
       for (int k = 0; k < 5; ++k) sh.e[k] = 0;
@@ -618,81 +730,54 @@ __global__ void __launch_bounds__(kFxThreads, 2) npr_kernel(const __grid_constan
       issue_loads<kFxThreads>(a, h + gridDim.x, reinterpret_cast<double2 *>(gs),
                               reinterpret_cast<double2 *>(ut));
     if (bad) continue;  // the same in every thread
+    // cut into digits: with 256 (1 + 512 + ... + 512^5) added, the digits are
+    // the value's 9-bit fields less 256; 1024 + field is an FP16 bit pattern
 #pragma unroll 1
     for (int i = tid; i < 2 * 2304; i += kFxThreads) {
-      const int k = i >= 2304, j = i - k * 2304;
-      int4 *p = k ? qs + j : ps + (j / 144) * kFxRow + j % 144;
-      const longlong2 v = *reinterpret_cast<const longlong2 *>(p);
+      const int k = i >= 2304;
+      const longlong2 v = pq[i];
       const int s = k ? sc[1] : sc[0];
       const long long half = s > 0 ? 1ll << (s - 1) : 0;
-      *p = fx_word((v.x + half) >> s, (v.y + half) >> s);
-    }
-    __syncthreads();
-    Wide w[9];
+      constexpr long long bias = 256ll * (1ll + 512 + (1ll << 18) + (1ll << 27) + (1ll << 36) + (1ll << 45));
+      const unsigned long long re = (unsigned long long)(((v.x + half) >> s) + bias);
+      const unsigned long long im = (unsigned long long)(((v.y + half) >> s) + bias);
+      const int j = i - k * 2304;
+      __half2 *dst = reinterpret_cast<__half2 *>(pd + k * (256 * kRowHalfs) + (j / 9) * kRowHalfs) + j % 9;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) w[k] = {0, 0, 0, 0};
-    if (mine) fx_contract<SLICES>(ps, qs, op, a1, a3, slice, w);
-    // add the slices; afterwards every lane of a group holds the sums, as
-    // 4 (re + rl 2^-FX_LOW): the sum of all slices may need 65 bits
-    long long re[9], im[9];
-    unsigned rl[9], il[9];
-    constexpr int mask = (1 << FX_LOW) - 1;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const long long vr = w[k].hr + (w[k].mr >> FX_LOW), vi = w[k].hi + (w[k].mi >> FX_LOW);
-      re[k] = vr >> 2;
-      rl[k] = (((unsigned)vr & 3) << (FX_LOW - 2)) | (((unsigned)w[k].mr & mask) >> 2);
-      im[k] = vi >> 2;
-      il[k] = (((unsigned)vi & 3) << (FX_LOW - 2)) | (((unsigned)w[k].mi & mask) >> 2);
-#pragma unroll
-      for (int d = 1; d < SLICES; d <<= 1) {
-        re[k] += __shfl_xor_sync(0xffffffffu, re[k], d);
-        im[k] += __shfl_xor_sync(0xffffffffu, im[k], d);
-        rl[k] += __shfl_xor_sync(0xffffffffu, rl[k], d);
-        il[k] += __shfl_xor_sync(0xffffffffu, il[k], d);
+      for (int d = 0; d < kDigits; ++d) {  // from the top
+        const int at = kDigitBits * (kDigits - 1 - d);
+        const unsigned mr = d ? 511u : 1023u;  // the top field may reach 512
+        const unsigned w = ((unsigned)(re >> at) & mr) | (((unsigned)(im >> at) & mr) << 16) | 0x64006400u;
+        dst[9 * d] = __hsub2(*reinterpret_cast<const __half2 *>(&w), __floats2half2_rn(1280.f, 1280.f));
       }
     }
-    if (mine) {
-      // units: P 2^(eu + e4 + e1 - kLinkBits - 2 kPropBits + ... + s), Q the
-      // same with flavours 2, 3; the sums are in 2^(2 FX_LOW) of their product
-      constexpr int vb = kMidBits + kPropBits - 2 * FX_LOW + 2;  // bits of |v| at scale 1
-      const int ex = 2 * eu + (e[0] + e[1] + e[2] + e[3] - 4 * 1022) + sc[0] + sc[1] - 2 * vb +
-                     2 * FX_LOW + 2;
-      const double unit = __hiloint2double((ex + 1023) << 20, 0);
-#pragma unroll
-      for (int r = 0; r < kOwn; ++r) {
-        const int k = r * SLICES + slice;
-        long long vr = re[0], vi = im[0];
-        unsigned lr = rl[0], li = il[0];
-#pragma unroll
-        for (int j = r * SLICES; j < (r + 1) * SLICES && j < 9; ++j)
-          if (j == k) {
-            vr = re[j];
-            vi = im[j];
-            lr = rl[j];
-            li = il[j];
-          }
-        if (k < 9) {
-          // low part through the bits of 2^52 + l: subtract its 2^52 / 2^27 from the high part
-          const double dr = fma(__hiloint2double(0x43300000, (int)lr), 1.0 / (1 << FX_LOW),
-                                (double)(vr - (1ll << (52 - FX_LOW))));
-          const double di = fma(__hiloint2double(0x43300000, (int)li), 1.0 / (1 << FX_LOW),
-                                (double)(vi - (1ll << (52 - FX_LOW))));
-          if (a.out_hc)
-            a.out_hc[(long)h * a.hc_stride + iop * 81 + 27 * a1 + 9 * (k % 3) + 3 * a3 + k / 3] =
-                make_double2(dr * unit, di * unit);
-          tot[r].x = fma(dr, unit, tot[r].x);
-          tot[r].y = fma(di, unit, tot[r].y);
+    // units: P 2^(eu + e4 + e1 - vb + s), Q the same with flavours 2, 3; the
+    // sums are in 512^7 of their product
+    constexpr int vb = kMidBits + kPropBits - 2 * FX_LOW + 2;  // bits of |v| at scale 1
+    const int ex = 2 * eu + (e[0] + e[1] + e[2] + e[3] - 4 * 1022) + sc[0] + sc[1] - 2 * vb + 7 * kDigitBits;
+    const double unit = __hiloint2double((ex + 1023) << 20, 0);
+    __syncthreads();
+    // operator op's products while op - 1's are added, C alternating between
+    // two buffers
+#pragma unroll 1
+    for (int op = 0; op <= a.nops; ++op) {
+      if (op < a.nops) digit_products(pd_s, qd_s, a.ops[op], cm + (op & 1) * kCFloats, mt, nt, ntiles);
+      if (op > 0 && tid < 352) {  // whole warps with outputs
+        long long hi, lo;
+        digit_sum(cm + ((op - 1) & 1) * kCFloats, ra, rb, hi, lo);
+        // parts 0..3: re re, re im, im re, im im; part 0 becomes re re - im im,
+        // part 1 re im + im re
+        const long long hx = __shfl_xor_sync(0xffffffffu, hi, 3), lx = __shfl_xor_sync(0xffffffffu, lo, 3);
+        hi += part == 0 ? -hx : hx;
+        lo += part == 0 ? -lx : lx;
+        if (mine && part < 2) {
+          const double d = fma((double)lo, 1.0 / (1 << 27), (double)hi);
+          const int at = (op - 1) * 81 + o;
+          if (a.out_hc) reinterpret_cast<double *>(a.out_hc + (long)h * a.hc_stride + at)[part] = d * unit;
+          sum[2 * at + part] = fma(d, unit, sum[2 * at + part]);
         }
       }
-    }
-  }
-  if (mine) {
-#pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-      const int k = r * SLICES + slice;
-      if (k < 9)
-        a.partial[((long)blockIdx.x * a.nops + iop) * 81 + 27 * a1 + 9 * (k % 3) + 3 * a3 + k / 3] = tot[r];
+      __syncthreads();
     }
   }
 }
@@ -753,23 +838,11 @@ extern "C" int npr_four_fermion(sq_ctx *ctx, const int dims[4], const double *li
 
   cudaSetDevice(ctx->device);
   cudaStream_t st = stream ? (cudaStream_t)stream : cudaStreamLegacy;  // NULL: default stream
-  // 2 to 16 slices of the sum over A per output tile: as many as the 288
-  // threads hold for the operators of a group (9 tiles each)
-  auto kernel_for = [](int n) {
-    return n <= 2 ? npr_kernel<16> : n <= 4 ? npr_kernel<8> : n <= 8 ? npr_kernel<4> : npr_kernel<2>;
-  };
   SQ_CUDA_TRY(cudaFuncSetAttribute(npr_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kSmemBytes));
-  const int first = std::min(kMaxOps, nops), rest = nops % kMaxOps;
-  for (int n : {first, rest})
-    if (n > 0)
-      SQ_CUDA_TRY(cudaFuncSetAttribute(kernel_for(n), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kFxSmem));
-  int per_sm = 0;
-  SQ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_for(first), kFxThreads,
-                                                            kFxSmem));
-  if (per_sm < 1) per_sm = 1;
-  const int grid = (int)std::min<long>(a.nhc, (long)per_sm * ctx->sms);
+  SQ_CUDA_TRY(cudaFuncSetAttribute(npr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kFxSmem));
+  const int grid = (int)std::min<long>(a.nhc, ctx->sms);  // one CTA per SM
   void *partial = nullptr;
   const size_t partial_b = sizeof(double2) * (size_t)grid * kMaxOps * 81;
   SQ_CUDA_TRY(cudaMallocAsync(&partial, partial_b + 16 + (size_t)a.nhc, st));
@@ -794,8 +867,8 @@ extern "C" int npr_four_fermion(sq_ctx *ctx, const int dims[4], const double *li
     }
     a.out_hc = out_hc_dev ? reinterpret_cast<double2 *>(out_hc_dev) + 81L * g0 : nullptr;
     const int nitems = a.nops * 81;
-    kernel_for(a.nops)<<<grid, kFxThreads, kFxSmem, st>>>(a);
-    npr_fp64_kernel<<<std::min(grid, ctx->sms), kThreads, kSmemBytes, st>>>(a);
+    npr_kernel<<<grid, kFxThreads, kFxSmem, st>>>(a);
+    npr_fp64_kernel<<<grid, kThreads, kSmemBytes, st>>>(a);
     e = cudaGetLastError();
     if (e == cudaSuccess) {
       npr_sum_kernel<<<(nitems + 255) / 256, 256, 0, st>>>(
