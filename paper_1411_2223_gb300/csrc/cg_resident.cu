@@ -348,7 +348,6 @@ int launch_split(const ResidentArgs &a, int block, int lanes, cudaStream_t st) {
 static size_t barrier_bytes(const sq_ctx *ctx) {
   return (256 + sizeof(double) * 2 * ctx->sms + 255) / 256 * 256;
 }
-size_t cg_resident_bytes(const sq_ctx *ctx, size_t fb) { return barrier_bytes(ctx) + fb; }
 
 // One site per thread of one block per SM (77824 sites per parity on 152 SMs)
 // is as far as the resident form goes; it is the faster one up to there, in
@@ -357,13 +356,21 @@ size_t cg_resident_bytes(const sq_ctx *ctx, size_t fb) { return barrier_bytes(ct
 //   FP32           21.7  10.1  23.1  10.4  28.5  19.4  32.2  26.0  42.1  34.8
 //   16-bit         22.1  14.4  24.6  14.2  27.1  18.6  29.0  22.1  36.9  32.3
 //   FP64           41.5  20.1  54.1  26.7  65.4  43.0  68.2  54.2  86.4  78.0
-// (whole solves over their iterations, reliable updates included).  With two
+// (whole solves over their iterations, reliable updates included, at one
+// thread per site then: with a site's directions on four warps, 2048 sites
+// take 9.5 in FP32 and 12.6 in 16-bit, 20736 take 19.2 and 18.0).  With two
 // rounds per thread it loses: 50.5 against 42.1 at 65536 sites, 170 against
 // 114 at 256000, as the SMs' last round is part empty.
+size_t cg_resident_bytes(const sq_ctx *ctx, int vh, int nrhs, int prec, size_t fb) {
+  if (nrhs != 1 || vh > 512 * ctx->sms) return 0;
+  const bool merged = prec == PREC_F32 && lanes_per_site(vh, ctx->sms) == 4;
+  return barrier_bytes(ctx) + (merged ? fb : 0);
+}
+
 int cg_resident_block(const CGWork *w) {
   const sq_ctx *ctx = w->ctx;
   const int vh = w->gf->g.vh;
-  if (w->nrhs != 1 || vh > 512 * ctx->sms) return 0;
+  if (w->resident == nullptr) return 0;  // too large, or no memory for it
   if (w->prec == PREC_F64 && !w->gf->scales(PREC_F64, w->recon).fixed) return 0;
   int coop = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop)

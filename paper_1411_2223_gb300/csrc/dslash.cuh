@@ -871,7 +871,10 @@ inline size_t dslash_smem_bytes(int prec, int recon, int nr, int block) {
 // GATED: in dslash_gated_kernel, whose PLAIN form gathers x64 + xs.
 // One work item of the kernel: RHS tile blk % ntiles of the blockDim.x
 // sites from (blk / ntiles) * blockDim.x on.  A return ends the item.
-template <int PREC, int RECON, int NR, int MODE, int OUTP, bool GATED>
+// SPLIT (one system per item): blocks of 128 threads and items of 32 sites;
+// warp k takes direction k of them, and warp 0 adds the four sums and goes on
+// alone, so that the reductions' warps are those of the unsplit form.
+template <int PREC, int RECON, int NR, int MODE, int OUTP, bool GATED, bool SPLIT = false>
 __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned blk) {
   using R = typename AccumType<PREC>::R;
   const Geom &g = a.g;
@@ -880,7 +883,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
   // order, so the tiles after the first find that range's links in L2.
   const int ntiles = (a.nrhs + NR - 1) / NR;
   const int tile = blk % ntiles;
-  const int i = (blk / ntiles) * blockDim.x + threadIdx.x;
+  const int i = SPLIT ? (blk / ntiles) * 32 + (threadIdx.x & 31) : (blk / ntiles) * blockDim.x + threadIdx.x;
   const int r0 = tile * NR;
   LinkScales ls = a.ls;
   ls.keep = tile < ntiles - 1;  // a later tile of this site range reads the links again
@@ -970,6 +973,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
       active[r] = (r0 + r < a.nrhs) && slot_active(a.slots + r0 + r, a.gate);
       any_here |= active[r];
     }
+    if constexpr (SPLIT) active[0] = any_here = __syncthreads_or(any_here) != 0;  // one decision a block
     if (!any_here) {
       if constexpr (kStaged) cp_async_wait<0>();  // no copy outlives its thread
       return;
@@ -984,6 +988,8 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
   Vec3<R> acc[NR];
 #pragma unroll
   for (int r = 0; r < NR; ++r) zero(acc[r]);
+  constexpr int IN = GATED && MODE == MODE_PLAIN ? IN_XS : IN_HALF;  // RECON_FIXED
+  bool odd = false;
 
   if (valid) {
     const SiteCoords sc = site_coords(g, a.out_parity, i);
@@ -993,7 +999,8 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
       multi_hops<RECON, NR, MODE, kEarly>(a, ls, sc, i, r0, active, acc, dyn_smem, vbuf);
       if constexpr (EpiStage<MODE, RECON, NR>::V > 0) cp_async_wait<0>();
     } else if constexpr (RECON == RECON_FIXED) {
-      fixed_hops<NR, MODE, GATED && MODE == MODE_PLAIN ? IN_XS : IN_HALF>(a, ls, sc, i, r0, active, acc);
+      if constexpr (SPLIT) fixed_hops<NR, MODE, IN>(a, ls, sc, i, r0, active, acc, threadIdx.x / 32, 4, &odd);
+      else fixed_hops<NR, MODE, IN>(a, ls, sc, i, r0, active, acc);
     } else if constexpr (PREC == PREC_F64 && NR == 1) {
       pair_hops<PREC, RECON, NR, MODE>(a, ls, sc, i, r0, active, acc);
     } else {
@@ -1033,6 +1040,40 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
           }
         }
       }
+    }
+  }
+
+  if constexpr (SPLIT) {
+    __shared__ double part[3][6][32];
+    __shared__ bool part_odd[3][32];
+    const int dir = threadIdx.x / 32, lane = threadIdx.x & 31;
+    if (dir > 0) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        part[dir - 1][2 * c][lane] = acc[0].c[c].x;
+        part[dir - 1][2 * c + 1][lane] = acc[0].c[c].y;
+      }
+      part_odd[dir - 1][lane] = odd;
+    }
+    __syncthreads();
+    if (dir == 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          acc[0].c[c].x += part[k][2 * c][lane];
+          acc[0].c[c].y += part[k][2 * c + 1][lane];
+        }
+        odd |= part_odd[k][lane];
+      }
+    }
+    __syncthreads();  // the next item writes them again
+    if (dir > 0) return;
+    if (odd) {
+      double o[6];
+      fixed_site_fp64<MODE, IN>(a, i, r0, o);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[0].c[c] = make_double2(o[2 * c], o[2 * c + 1]);
     }
   }
 
@@ -1287,7 +1328,7 @@ constexpr int GATED_BLOCKS_PER_SM = 3;
 // taken by block k % gridDim.x.  An empty launch costs one wave of blocks,
 // not a block per item, and when some systems need an update every block
 // works on theirs.
-template <int RECON, int NR, int MODE, int OUTP>
+template <int RECON, int NR, int MODE, int OUTP, bool SPLIT = false>
 __global__ void __launch_bounds__(DslashBounds<PREC_F64, NR>::threads,
                                   NR == 1 ? GATED_BLOCKS_PER_SM : DslashBounds<PREC_F64, NR>::min_blocks)
 dslash_gated_kernel(const __grid_constant__ DslashArgs a) {
@@ -1295,9 +1336,10 @@ dslash_gated_kernel(const __grid_constant__ DslashArgs a) {
   const int ntiles = (a.nrhs + NR - 1) / NR;
   const unsigned long long act = active_tiles<NR>(a, ntiles);
   const int nact = __popcll(act);
-  const int n = nact * ((a.g.vh + (int)blockDim.x - 1) / (int)blockDim.x);
+  const int sites = SPLIT ? 32 : (int)blockDim.x;
+  const int n = nact * ((a.g.vh + sites - 1) / sites);
   for (int k = blockIdx.x; k < n; k += gridDim.x)
-    dslash_item<PREC_F64, RECON, NR, MODE, OUTP, true>(a, (k / nact) * ntiles + nth_bit(act, k % nact));
+    dslash_item<PREC_F64, RECON, NR, MODE, OUTP, true, SPLIT>(a, (k / nact) * ntiles + nth_bit(act, k % nact));
   griddep_launch_dependents();
 }
 

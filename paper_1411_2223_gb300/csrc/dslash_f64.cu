@@ -11,12 +11,31 @@ int launch_dslash_f64(int recon, int nr, int mode, int outp, const DslashArgs &a
   const bool fixed = a.ls.fixed;
   if (fixed) recon = RECON_FIXED;
   const bool gated = a.max_grid > 0 && (mode == MODE_PLAIN || mode == MODE_RESID) && recon != 12;
+  // One system on a small lattice: a thread per site leaves most of the chip
+  // idle through 16 hops in series, so a site's directions go to four warps.
+  // Whole solves, us, launched whole against split (FP32 / 16-bit; sites per
+  // parity): 2048: 1675 -> 1575 / 2400 -> 2106; 20736: 3618 -> 3576 / 3959 ->
+  // 3836; at 65536, where the grid is full either way, 6402 -> 6540.  Batches
+  // do not gain (4 systems of 20736: 7670 -> 7735).  The line is drawn at two
+  // items of 32 sites per block of the grid.
+  const bool split = gated && fixed && nr == 1 && a.nrhs == 1 &&
+                     dslash_items(a.g, 1, 1, 32) <= 2 * a.max_grid;
+  if (split) {
+    block = 128;
+    grid.x = dslash_items(a.g, 1, 1, 32);
+  }
   if (gated && grid.x > (unsigned)a.max_grid) grid.x = a.max_grid;
 #define SQ_K(RC, NR, MODE, OUTP) \
   if (recon == RC && nr == NR && mode == MODE && outp == OUTP) { \
     return launch_pdl(dslash_kernel<PREC_F64, RC, NR, MODE, OUTP>, grid, dim3(block), 0, st, a) == \
                    cudaSuccess ? 0 : -1; \
   }
+#define SQ_S(MODE, OUTP) \
+  if (split && mode == MODE && outp == OUTP) \
+    return launch_pdl(dslash_gated_kernel<RECON_FIXED, 1, MODE, OUTP, true>, grid, dim3(block), 0, st, \
+                      a) == cudaSuccess ? 0 : -1;
+  SQ_S(MODE_PLAIN, PREC_F64) SQ_S(MODE_RESID, PREC_F64) SQ_S(MODE_RESID, PREC_F32) SQ_S(MODE_RESID, PREC_I16)
+#undef SQ_S
 #define SQ_G(NR, MODE, OUTP) \
   if (gated && nr == NR && mode == MODE && outp == OUTP) { \
     auto kern = fixed ? dslash_gated_kernel<RECON_FIXED, NR, MODE, OUTP> \

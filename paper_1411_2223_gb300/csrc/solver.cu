@@ -62,12 +62,17 @@ int cg_work_create(sq_ctx *ctx, GaugeField *gf, int prec, int recon, int nrhs, C
   size_t sizes[] = {w->f64_fb * nrhs, w->f64_fb * nrhs, w->f64_fb * nrhs, w->fb * nrhs,
                     w->fb * nrhs,     w->fb * nrhs,     w->xs_fb * nrhs,
                     sizeof(SlotState) * nrhs, sizeof(double) * 4 * w->partial_stride,
-                    sizeof(unsigned) * 4 * w->counter_stride, nrhs == 1 ? cg_resident_bytes(ctx, w->fb) : 256};
+                    sizeof(unsigned) * 4 * w->counter_stride,
+                    cg_resident_bytes(ctx, g.vh, nrhs, prec, w->fb)};
   char **ptrs[] = {&w->x64, &w->b64, &w->t64, &w->r, &w->p, &w->t, &w->xs};
   size_t total = 0;
   for (size_t s : sizes) total += s;
   {
     std::lock_guard<std::mutex> lk(ctx->mu);
+    if (ctx->in_use + total > ctx->budget) {  // the launched kernels need less
+      total -= sizes[10];
+      sizes[10] = 0;
+    }
     if (ctx->in_use + total > ctx->budget) return SQ_ERR_OOM;
     ctx->in_use += total;
   }
@@ -77,8 +82,10 @@ int cg_work_create(sq_ctx *ctx, GaugeField *gf, int prec, int recon, int nrhs, C
   SQ_CUDA_TRY(cudaMalloc((void **)&w->slots_d, sizes[7]));
   SQ_CUDA_TRY(cudaMalloc((void **)&w->partial, sizes[8]));
   SQ_CUDA_TRY(cudaMalloc((void **)&w->counters, sizes[9]));
-  SQ_CUDA_TRY(cudaMalloc(&w->resident, sizes[10]));
-  SQ_CUDA_TRY(cudaMemset(w->resident, 0, sizes[10]));
+  if (sizes[10] > 0) {
+    SQ_CUDA_TRY(cudaMalloc(&w->resident, sizes[10]));
+    SQ_CUDA_TRY(cudaMemset(w->resident, 0, sizes[10]));
+  }
   SQ_CUDA_TRY(cudaMemset(w->counters, 0, sizes[9]));
   SQ_CUDA_TRY(cudaMemset(w->partial, 0, sizes[8]));
   // vectors start zeroed so no kernel reads NaN garbage from padding

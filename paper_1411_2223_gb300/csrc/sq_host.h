@@ -150,7 +150,7 @@ int cg_run_resident(CGWork *w, cudaStream_t st);
 // launch (a few ms at most, so that other streams' kernels get in between),
 // and its block for a workspace it is the faster form for (else 0).
 constexpr int RESIDENT_STEPS = 128;
-size_t cg_resident_bytes(const sq_ctx *ctx, size_t fb);
+size_t cg_resident_bytes(const sq_ctx *ctx, int vh, int nrhs, int prec, size_t fb);
 int cg_resident_block(const CGWork *w);
 int cg_enqueue_resident(CGWork *w, const DslashArgs &norm, const DslashArgs &update,
                         cudaStream_t st);

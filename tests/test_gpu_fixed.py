@@ -189,3 +189,28 @@ def test_dirac_apply_gathers_from_the_whole_lattice(sq, dims, antiperiodic):
             assert rel(got[~bad], want[~bad]) <= 1e-15
         finally:
             sq.gauge_free(gid)
+
+
+# around the size up to which a site's directions go to four warps (29184
+# sites per parity on 152 SMs), whole and part warps of sites
+@pytest.mark.parametrize('prec', ['f32', 'i16'])
+@pytest.mark.parametrize('dims', [(2, 2, 2, 2), (6, 2, 10, 4), (12, 14, 14, 24), (16, 16, 16, 16)])
+def test_reliable_updates_of_one_system(sq, dims, prec):
+    """The residual a solve reports is its last reliable update's: it is the
+    oracle's, to the FP64 rounding of A x (|x| <= 4 |b|, |A| of order 10: some
+    1e-14, with room 1e-12), also from a guess outside the fixed-point range."""
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    b = synth.gaussian_source(vh, 11)
+    tiny = np.zeros_like(b)
+    tiny[::7] = 1e-300
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        for x0 in (None, tiny):
+            x, st = sq.cg_solve(gid, b, 0.5, 1e-9, precision=prec, x0=x0)
+            assert st['status'] == 0
+            true = oracle.true_residual(dims, fat, lng, 0.5, b, x)
+            assert true <= 1e-9
+            assert abs(st['true_residual'] - true) <= 1e-12
+    finally:
+        sq.gauge_free(gid)
