@@ -50,7 +50,9 @@ __global__ void __launch_bounds__(256, S == PREC_F64 ? 4 : 8) cg_xpay_kernel(Vec
 // the block sums in order and runs finish_alpha (KIND 0: after the D_oe
 // kernel, the sum is <p, A p>) or finish_update (KIND 1: after the D_eo
 // kernel, the sum is |r|^2).  Systems the Dslash kernel skipped (not
-// running) are skipped here too.  Launched with programmatic stream
+// running) are skipped here too.  SHIFTS: multi-shift CG; the warp that sums
+// takes the shifts' steps as well, a lane each (in series, their FP64 divides
+// are on the iteration's critical path).  Launched with programmatic stream
 // serialization, it lets the next Dslash kernel launch -- and prefetch its
 // links -- while it adds.
 constexpr int FINISH_THREADS = 256;
@@ -60,7 +62,7 @@ constexpr int FINISH_BLOCKS = 16;
 // the groups of 32 warp partials, whose sum slots hold the block sums.
 inline int finish_blocks(const Geom &g) { return g.ngroups < FINISH_BLOCKS ? g.ngroups : FINISH_BLOCKS; }
 
-template <int KIND>
+template <int KIND, bool SHIFTS>
 __global__ void __launch_bounds__(FINISH_THREADS) cg_finish_kernel(VecArgs a) {
   __shared__ double smem[FINISH_THREADS / 32];
   griddep_wait();
@@ -78,19 +80,30 @@ __global__ void __launch_bounds__(FINISH_THREADS) cg_finish_kernel(VecArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) smem[warp] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (warp != 0) return;
+  bool last = false;
+  double sum = 0.0;
+  if (lane == 0) {
     double bs = 0.0;
 #pragma unroll
     for (int w = 0; w < FINISH_THREADS / 32; ++w) bs += smem[w];
     p[n + j] = bs;  // the group-sum slots of this reduction instance
     unsigned *ticket = a.counter + (size_t)sys * ticket_stride(a.g);
-    if (atom_add_acq_rel(ticket, 1u) == (unsigned)(nb - 1)) {
-      double sum = 0.0;
+    last = atom_add_acq_rel(ticket, 1u) == (unsigned)(nb - 1);
+    if (last) {
       for (int b = 0; b < nb; ++b) sum += __ldcg(p + n + b);
       *ticket = 0;
       if (KIND == 0) finish_alpha(s, sum);
-      else finish_update(s, sum, a.checkpoint);
+      else if (!SHIFTS) finish_update(s, sum, a.checkpoint);
     }
+  }
+  if constexpr (SHIFTS) {  // the shifts' scalars, a lane each
+    last = __shfl_sync(0xffffffffu, last, 0);
+    sum = __shfl_sync(0xffffffffu, sum, 0);
+    if (!last) return;
+    __syncwarp();  // alpha
+    if (KIND == 1) finish_shift_update(s, a.shifts, a.nshift, sum, lane);
+    else if (lane < a.nshift) finish_shift_alpha(s, a.shifts[lane]);
   }
 }
 
@@ -204,8 +217,9 @@ int launch_cg_xpay(int prec, const VecArgs &a, cudaStream_t st) {
 int launch_cg_finish(int kind, const VecArgs &a, cudaStream_t st) {
   if (a.g.vh <= 0) return 0;
   const dim3 grid(finish_blocks(a.g), a.nrhs), block(FINISH_THREADS);
-  cudaError_t e = (kind == 0) ? launch_pdl(cg_finish_kernel<0>, grid, block, 0, st, a)
-                              : launch_pdl(cg_finish_kernel<1>, grid, block, 0, st, a);
+  auto kern = a.shifts ? (kind == 0 ? cg_finish_kernel<0, true> : cg_finish_kernel<1, true>)
+                       : (kind == 0 ? cg_finish_kernel<0, false> : cg_finish_kernel<1, false>);
+  const cudaError_t e = launch_pdl(kern, grid, block, 0, st, a);
   return e == cudaSuccess ? 0 : -1;
 }
 

@@ -13,8 +13,6 @@
 // Epilogues:
 //   MODE_PLAIN  out = D in
 //   MODE_MDAGM  out = m^2 p - D in               (second Dslash of A = m^2 - D_eo D_oe)
-//               + per-chunk partials of Re<p, out>, and the last block sets
-//               alpha = rr / <p, Ap> for every running system
 //   MODE_RESID  r = b - (m^2 x - D in), FP64     (reliable update: true residual)
 //               with x = x64 + xs folded into x64 first; r is written in the
 //               sloppy precision OUTP, + partials of |r|^2 and <r, p_sloppy>;
@@ -65,8 +63,6 @@ struct DslashArgs {
   const char *ps;
   size_t ps_fb;
   SlotState *slots;           // nullptr: no CG state (operator application only)
-  ShiftState *shifts;         // multi-shift CG: shifted systems updated with alpha
-  int nshift;
   double *partial;            // [value][rhs][chunk]
   unsigned *counter;
   int gate;
@@ -1089,11 +1085,9 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
       }
     }
   } else if constexpr (MODE == MODE_MDAGM) {
-    // Ap = m^2 p - 1/2 acc ; partial Re<p, Ap>
-    R dot[NR];
+    // Ap = m^2 p - 1/2 acc
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      dot[r] = 0;
       if (valid && active[r]) {
         const R m2 = (R)(a.slots ? a.slots[r0 + r].m2 : a.m2_const);
         Vec3<R> p;
@@ -1101,35 +1095,12 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
         else if constexpr (kStaged) p = epi_vec<MODE, RECON, NR>(dyn_smem, vbuf, r);
         else p = SpinorIO<PREC>::load(a.p + (size_t)(r0 + r) * a.p_fb, S, i);
         Vec3<R> o;
-        R d = 0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           o.c[c].x = fma(m2, p.c[c].x, R(-0.5) * acc[r].c[c].x);
           o.c[c].y = fma(m2, p.c[c].y, R(-0.5) * acc[r].c[c].y);
-          d = fma(p.c[c].x, o.c[c].x, d);
-          d = fma(p.c[c].y, o.c[c].y, d);
         }
         SpinorIO<PREC>::store(a.out + (size_t)(r0 + r) * a.out_fb, S, i, o);
-        dot[r] = d;
-      }
-    }
-    if (a.slots != nullptr && a.partial != nullptr && any_here) {
-      // <p, Ap> of every system of this tile; the warp completing the sums
-      // sets alpha for the tile's running systems
-      double *inst[NR];
-#pragma unroll
-      for (int r = 0; r < NR; ++r)
-        inst[r] = a.partial + (size_t)min(r0 + r, a.nrhs - 1) * red_stride(g);
-      double pap[NR];
-      if (warp_tree_reduce<NR>(dot, min(NR, a.nrhs - r0), inst, g, i,
-                               a.counter + (size_t)tile * ticket_stride(g), pap) &&
-          (threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          if (!active[r]) continue;
-          finish_alpha(a.slots + r0 + r, pap[r]);
-          if (a.shifts) finish_shift_alpha(a.slots + r0 + r, a.shifts, a.nshift);
-        }
       }
     }
   } else if constexpr (MODE == MODE_NORM) {

@@ -3,10 +3,15 @@
 // in the sloppy precision, followed by a batched mixed-precision refinement
 // of every shift started from its shifted solution.
 //
-// One iteration = four kernels: the base system's two Dslash (the second one
-// also yields alpha and the shifted alpha_i), ms_update (r -= alpha Ap,
-// |r|^2; beta, beta_i, per-shift convergence) and ms_xpay (x_i += alpha_i p_i,
-// p_i = zeta_i r + beta_i p_i for every shift).
+// One iteration = five kernels: the base system's two Dslash with the CG's
+// epilogues (the first sums <p, A p>, the second updates x and r in
+// registers), the finish kernel after each (alpha and the shifted alpha_i;
+// beta, beta_i and per-shift convergence, a lane per shift) and ms_xpay
+// (x_i += alpha_i p_i of the shifts, p_i = zeta_i r + beta_i p_i of all).  It
+// moves about 3290 bytes per site and iteration with 8 shifts, the bound of
+// the phase.  8 masses at 24^3 x 64, whole solve: 145.5 ms; with <p, A p>
+// summed in the second Dslash by tickets, A p stored, r updated by a kernel
+// of its own and the shifts' scalars in one thread it was 149.9 ms.
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -27,7 +32,7 @@ namespace {
 struct MsArgs {
   Geom g;
   int nshift, base;
-  char *r, *ap, *p, *x;     // r, Ap: 1 field; p, x: nshift fields
+  char *r, *p, *x;          // r: 1 field; p, x: nshift fields
   size_t fb, xfb;
   const char *b64;
   SlotState *bs;
@@ -82,40 +87,14 @@ __global__ void __launch_bounds__(256) ms_init_kernel(MsArgs a) {
   }
 }
 
-// r -= alpha Ap ; |r|^2 ; last block: finish_shift_update
-template <int S>
-__global__ void __launch_bounds__(256) ms_update_kernel(MsArgs a) {
-  using R = typename SpinorIO<S>::R;
-  if (a.bs->status != SLOT_RUNNING) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int St = a.g.stride;
-  double val[1] = {0.0};
-  if (i < a.g.vh) {
-    const R al = (R)a.bs->alpha;
-    Vec3<R> ap = SpinorIO<S>::load(a.ap, St, i);
-    Vec3<R> rv = SpinorIO<S>::load(a.r, St, i);
-    R n2 = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      rv.c[c].x = fma(-al, ap.c[c].x, rv.c[c].x);
-      rv.c[c].y = fma(-al, ap.c[c].y, rv.c[c].y);
-      n2 = fma(rv.c[c].x, rv.c[c].x, fma(rv.c[c].y, rv.c[c].y, n2));
-    }
-    SpinorIO<S>::store(a.r, St, i, rv);
-    val[0] = (double)n2;
-  }
-  double *const inst[1] = {a.partial};
-  double rr[1];
-  if (warp_tree_reduce<1>(val, 1, inst, a.g, i, a.counter, rr) && (threadIdx.x & 31) == 0)
-    finish_shift_update(a.bs, a.sh, a.nshift, rr[0]);
-}
-
-// x_i += alpha_i p_i ; p_i = zeta_i r + beta_i p_i ; the last block closes
-// the iteration (active <- cont, and a waiting base takes its final status).
+// x_i += alpha_i p_i (the base's x is updated with its r) ; p_i = zeta_i r +
+// beta_i p_i ; the last block closes the iteration (active <- cont, and a waiting base takes its final status).
 template <int S>
 __global__ void __launch_bounds__(256) ms_xpay_kernel(MsArgs a) {
   using R = typename SpinorIO<S>::R;
   constexpr int XP = (S == PREC_F64) ? PREC_F64 : PREC_F32;
+  griddep_wait();
+  griddep_launch_dependents();
   if (!ms_live(a.bs)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int St = a.g.stride;
@@ -125,9 +104,10 @@ __global__ void __launch_bounds__(256) ms_xpay_kernel(MsArgs a) {
     for (int k = 0; k < a.nshift; ++k) {
       const ShiftState &s = a.sh[k];
       const bool pc = (k == a.base) ? base_cont : (s.cont != 0 && base_cont);
-      if (!s.active && !pc) continue;
+      const bool ax = s.active && k != a.base;
+      if (!ax && !pc) continue;
       Vec3<R> p = SpinorIO<S>::load(a.p + k * a.fb, St, i);
-      if (s.active) {
+      if (ax) {
         const R al = (R)s.alpha;
         auto x = SpinorIO<XP>::load(a.x + k * a.xfb, St, i);
 #pragma unroll
@@ -171,11 +151,10 @@ int launch_prec(int prec, dim3 grid, cudaStream_t st, Args... args) {
 template <int S> struct InitL {
   static void run(dim3 g, cudaStream_t st, const MsArgs &a) { ms_init_kernel<S><<<g, 256, 0, st>>>(a); }
 };
-template <int S> struct UpdL {
-  static void run(dim3 g, cudaStream_t st, const MsArgs &a) { ms_update_kernel<S><<<g, 256, 0, st>>>(a); }
-};
 template <int S> struct XpayL {
-  static void run(dim3 g, cudaStream_t st, const MsArgs &a) { ms_xpay_kernel<S><<<g, 256, 0, st>>>(a); }
+  static void run(dim3 g, cudaStream_t st, const MsArgs &a) {
+    launch_pdl(ms_xpay_kernel<S>, g, dim3(256), 0, st, a);  // its error is read after the iteration
+  }
 };
 
 // Workspace of one multi-shift solve shape (cached per context).
@@ -184,7 +163,7 @@ struct MsWork {
   GaugeField *gf = nullptr;
   int prec = PREC_F32, recon = 18, nshift = 0, base = 0;
   size_t fb = 0, xfb = 0, f64_fb = 0, bytes = 0;
-  char *b64 = nullptr, *r = nullptr, *ap = nullptr, *t = nullptr, *p = nullptr, *x = nullptr;
+  char *b64 = nullptr, *r = nullptr, *t = nullptr, *p = nullptr, *x = nullptr;
   double *canon = nullptr;  // 2 * nshift canonical vectors: sources, solutions
   SlotState *bs_d = nullptr, *bs_h = nullptr;
   ShiftState *sh_d = nullptr, *sh_h = nullptr;
@@ -192,13 +171,13 @@ struct MsWork {
   unsigned *counters = nullptr;
   cudaGraphExec_t exec = nullptr;
   int exec_iters = 0, exec_kernels = 0;
-  DslashConfig cfg, cfg_mdagm;
+  DslashConfig cfg_norm, cfg_update;
 
   ~MsWork() {
     if (exec) cudaGraphExecDestroy(exec);
     if (bs_h) cudaFreeHost(bs_h);
     if (sh_h) cudaFreeHost(sh_h);
-    void *bufs[] = {b64, r, ap, t, p, x, canon, bs_d, sh_d, partial, counters};
+    void *bufs[] = {b64, r, t, p, x, canon, bs_d, sh_d, partial, counters};
     for (void *b : bufs)
       if (b) cudaFree(b);
     if (ctx) {
@@ -232,10 +211,10 @@ int ms_work_get(sq_ctx *ctx, GaugeField *gf, int gid, int prec, int recon, int n
   w->xfb = spinor_bytes(xs_prec(prec), g.stride);
   w->f64_fb = spinor_bytes(PREC_F64, g.stride);
   const size_t canon_b = (size_t)3 * g.vh * 16;
-  size_t sizes[] = {w->f64_fb, w->fb, w->fb, w->fb, w->fb * nshift, w->xfb * nshift,
+  size_t sizes[] = {w->f64_fb, w->fb, w->fb, w->fb * nshift, w->xfb * nshift,
                     2 * canon_b * nshift, sizeof(SlotState), sizeof(ShiftState) * nshift,
-                    sizeof(double) * red_stride(g), sizeof(unsigned) * (2 * ticket_stride(g) + 4)};
-  char **ptrs[] = {&w->b64, &w->r, &w->ap, &w->t, &w->p, &w->x};
+                    sizeof(double) * red_stride(g), sizeof(unsigned) * (ticket_stride(g) + 4)};
+  char **ptrs[] = {&w->b64, &w->r, &w->t, &w->p, &w->x};
   size_t total = 0;
   for (size_t s : sizes) total += s;
   {
@@ -245,21 +224,21 @@ int ms_work_get(sq_ctx *ctx, GaugeField *gf, int gid, int prec, int recon, int n
   }
   w->ctx = ctx;
   w->bytes = total;
-  for (int k = 0; k < 6; ++k) {
+  for (int k = 0; k < 5; ++k) {
     SQ_CUDA_TRY(cudaMalloc((void **)ptrs[k], sizes[k]));
     SQ_CUDA_TRY(cudaMemset(*ptrs[k], 0, sizes[k]));
   }
-  SQ_CUDA_TRY(cudaMalloc((void **)&w->canon, sizes[6]));
-  SQ_CUDA_TRY(cudaMalloc((void **)&w->bs_d, sizes[7]));
-  SQ_CUDA_TRY(cudaMalloc((void **)&w->sh_d, sizes[8]));
-  SQ_CUDA_TRY(cudaMalloc((void **)&w->partial, sizes[9]));
-  SQ_CUDA_TRY(cudaMalloc((void **)&w->counters, sizes[10]));
-  SQ_CUDA_TRY(cudaMemset(w->counters, 0, sizes[10]));
+  SQ_CUDA_TRY(cudaMalloc((void **)&w->canon, sizes[5]));
+  SQ_CUDA_TRY(cudaMalloc((void **)&w->bs_d, sizes[6]));
+  SQ_CUDA_TRY(cudaMalloc((void **)&w->sh_d, sizes[7]));
+  SQ_CUDA_TRY(cudaMalloc((void **)&w->partial, sizes[8]));
+  SQ_CUDA_TRY(cudaMalloc((void **)&w->counters, sizes[9]));
+  SQ_CUDA_TRY(cudaMemset(w->counters, 0, sizes[9]));
   // the clears are on the legacy stream, the solver's kernels on streams that
   // do not wait for it
   SQ_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
-  SQ_CUDA_TRY(cudaMallocHost((void **)&w->bs_h, sizes[7]));
-  SQ_CUDA_TRY(cudaMallocHost((void **)&w->sh_h, sizes[8]));
+  SQ_CUDA_TRY(cudaMallocHost((void **)&w->bs_h, sizes[6]));
+  SQ_CUDA_TRY(cudaMallocHost((void **)&w->sh_h, sizes[7]));
   *out = w.get();
   g_ms[key] = std::move(w);
   return SQ_OK;
@@ -271,7 +250,6 @@ MsArgs ms_args(MsWork *w) {
   a.nshift = w->nshift;
   a.base = w->base;
   a.r = w->r;
-  a.ap = w->ap;
   a.p = w->p;
   a.x = w->x;
   a.fb = w->fb;
@@ -299,24 +277,34 @@ int ms_enqueue_iteration(MsWork *w, cudaStream_t st) {
   a.ls = w->gf->scales(w->prec, w->recon, 1);
   a.in = pb;
   a.out = w->t;
-  if (launch_dslash(w->prec, w->recon, 1, MODE_PLAIN, w->prec, a, w->cfg.block, st)) return SQ_ERR_ARG;
+  a.partial = w->partial;
+  a.counter = w->counters;
+  if (launch_dslash(w->prec, w->recon, 1, MODE_NORM, w->prec, a, w->cfg_norm.block, st)) return SQ_ERR_ARG;
+  VecArgs f;
+  std::memset(&f, 0, sizeof(f));
+  f.g = g;
+  f.nrhs = 1;
+  f.slots = w->bs_d;
+  f.partial = w->partial;
+  f.counter = w->counters;
+  f.shifts = w->sh_d;
+  f.nshift = w->nshift;
+  if (launch_cg_finish(0, f, st)) return SQ_ERR_ARG;  // alpha, alpha_i
   DslashArgs b = a;
   b.out_parity = 0;
   b.links = w->gf->link_ptr(w->prec, w->recon, 0);
   b.in = w->t;
-  b.out = w->ap;
+  b.out = w->r;
   b.p = pb;
-  b.partial = w->partial;
-  b.counter = w->counters + ticket_stride(g) + 1;
-  b.shifts = w->sh_d;
-  b.nshift = w->nshift;
-  if (launch_dslash(w->prec, w->recon, 1, MODE_MDAGM, w->prec, b, w->cfg_mdagm.block, st))
+  b.xs = w->x + (size_t)w->base * w->xfb;
+  b.xs_prec = xs_prec(w->prec);
+  if (launch_dslash(w->prec, w->recon, 1, MODE_UPDATE, w->prec, b, w->cfg_update.block, st))
     return SQ_ERR_ARG;
+  if (launch_cg_finish(1, f, st)) return SQ_ERR_ARG;  // beta, beta_i
   dim3 grid((g.vh + 255) / 256);
   MsArgs m = ms_args(w);
-  if (launch_prec<UpdL>(w->prec, grid, st, m)) return SQ_ERR_ARG;
   if (launch_prec<XpayL>(w->prec, grid, st, m)) return SQ_ERR_ARG;
-  ctx->launches += 4;
+  ctx->launches += 5;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_cuda_error(e, "multi-shift launch", __FILE__, __LINE__);
@@ -422,8 +410,8 @@ extern "C" int cg_solve_multishift(sq_ctx *ctx, int gauge_id, const double *src,
     w->exec = nullptr;
   }
   w->base = base;
-  w->cfg = tuned_dslash(ctx, *gf, o.precision, o.long_recon, 1, MODE_PLAIN, st);
-  w->cfg_mdagm = tuned_dslash(ctx, *gf, o.precision, o.long_recon, 1, MODE_MDAGM, st);
+  w->cfg_norm = tuned_dslash(ctx, *gf, o.precision, o.long_recon, 1, MODE_NORM, st);
+  w->cfg_update = tuned_dslash(ctx, *gf, o.precision, o.long_recon, 1, MODE_UPDATE, st);
 
   // sources: nshift canonical copies of b (device); solutions follow them
   double *csrc = w->canon, *cx = w->canon + 2 * vec * nshift;

@@ -141,6 +141,8 @@ static VecArgs vec_args(CGWork *w, int region) {
   a.partial = w->partial + region * w->partial_stride;
   a.counter = w->counters + region * w->counter_stride;
   a.checkpoint = 0;
+  a.shifts = nullptr;
+  a.nshift = 0;
   return a;
 }
 

@@ -22,6 +22,8 @@ struct VecArgs {
   double *partial;
   unsigned *counter;
   int checkpoint;     // finish after the update: a reliable update may follow this iteration
+  ShiftState *shifts; // multi-shift CG (one system): its shifts, or null
+  int nshift;         // at most 32
 };
 
 // Launch with programmatic stream serialization (the kernel must call

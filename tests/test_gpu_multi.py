@@ -300,3 +300,24 @@ def test_64_system_batch_matches_oracle(sq):
             assert oracle.true_residual(dims, fat, lng, masses[j], srcs[j], xs[j]) <= tol
     finally:
         sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('prec', ['f64', 'f32', 'i16'])
+@pytest.mark.parametrize('nshift', [2, 16])
+def test_multishift_any_order_of_masses(sq, prec, nshift):
+    """The most shifts a call takes, the lightest mass not first (its x is
+    updated with r, the others' with p), on a lattice of whole and part warps."""
+    dims = (6, 2, 10, 4)
+    fat, lng = gauge(dims, 0.25, 0)
+    b = synth.gaussian_source(oracle.volume(dims) // 2, 3)
+    masses = [0.05 * 1.15 ** ((5 * k + 3) % nshift) for k in range(nshift)]
+    assert min(masses) != masses[0]
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        xs, stats, status = sq.cg_solve_multishift(gid, b, masses, 1e-9, precision=prec)
+        assert status == 0
+        for m, x, s in zip(masses, xs, stats):
+            assert s['true_residual'] <= 1e-9
+            assert oracle.true_residual(dims, fat, lng, m, b, x) <= 1e-9
+    finally:
+        sq.gauge_free(gid)
