@@ -36,7 +36,7 @@
 //   - step 4, four fifths of the work, on the tensor cores: P and Q, at one
 //     scale each, are cut into six signed 9-bit digits, which FP16 holds
 //     exactly, and the digits' products are summed over the 256 (A, C) by
-//     mma.sync with FP32 accumulators, exactly (256 256 256 = 2^24).
+//     tcgen05.mma into FP32 accumulators in TMEM, exactly (256 256 256 = 2^24).
 // A hypercube whose inputs or averaged links do not fit that form (infinities,
 // NaN, elements near the ends of FP64, links far from unitary) is marked there
 // and computed by npr_fp64_kernel in FP64.
@@ -335,20 +335,23 @@ __global__ void __launch_bounds__(kThreads, 1) npr_fp64_kernel(const NprArgs a) 
 // row 18 i + 2 (3 a1 + a4) + (0 re, 1 im) of the [108] x [256] matrix of p
 // digits and column 18 j + 2 (3 a3 + a2) + (0, 1) of the [256] x [108] matrix
 // of q digits give C = one 108 x 108 product per operator, of which the blocks
-// i + j <= 6 are needed (the others are below 2^-59 of the scales' product):
-// 75 of the 7 x 14 tiles of m16n8k16, 16 steps of k each.  The matrices lie in
-// shared memory by rows of k = (A, D) and (B, C) -- 240 bytes, so that the
-// eight rows an ldmatrix reads fall on different banks -- and an operator's
-// permutation D = C ^ t2, B = A ^ t1 is in the rows' addresses, its signs in an
-// XOR of the fragments.  The sums of digit pairs of one i + j are added as
-// integers, the seven of them to two 64-bit words, and these converted once.
+// i + j <= 6 are needed (the others are below 2^-59 of the scales' product).
+// It is 16 tcgen05.mma of M 128, N 112, K 16 by one thread, one per A: P's
+// digits stay as they were cut, in rows (A, D); Q's, in rows (B, C), are
+// brought from the last operator's order of C and signs to this one's in place
+// (an XOR of the row within 16, so pairs of rows swap), and B = A ^ t1 is in
+// the descriptors.  While the tensor cores work, the last operator's C is
+// added: the sums of digit pairs of one i + j as integers, the seven of them
+// to two 64-bit words, and these converted once.  The wait for the products is
+// bounded; a block in which one runs out returns NaN.
 //
 // 8 operators at 20^3 x 64: 37.2 ms with FP64 FMAs (their pipe 93 % busy),
 // 15.2 ms with the contraction on the integer units too (three mad.wide.s32
-// per real product, 32 lanes a clock and SM: 62 of its 147 thousand cycles per
-// hypercube at best), 9.8 ms here: about 40 thousand cycles up to the digits
-// and 7 thousand per operator, of which the tensor cores (938 multiply-adds a
-// clock and SM for mma.sync) take 2.6 and the ldmatrix reads 3.7.  Error of a
+// per real product, 32 lanes a clock and SM), 9.8 ms with mma.sync (7 thousand
+// cycles per operator, of which ldmatrix reads of the permuted rows 3.7),
+// 8.2 ms here.  About 40 thousand cycles per hypercube go to the steps up to
+// the digits (the integer multiply-adds alone are 10), 5 thousand to each
+// operator: reordering Q, and C from TMEM through shared memory.  Error of a
 // hypercube against long double 3.2e-16 to 3.6e-16, with FP64 FMAs (three per
 // complex term) 4.6e-16.
 struct FxC { Fx re, im; };
@@ -401,14 +404,20 @@ constexpr int kPropBits = FX_BITS, kLinkBits = 56;   // bits at the blocks' scal
 constexpr int kMidBits = 55;                         // ... of U G4 and U G2
 constexpr int kDigits = 6, kDigitBits = 9;
 constexpr int kPQBits = kDigits * kDigitBits - 1;    // P and Q: |v| <= 2^53
-constexpr int kRowHalfs = 120;                       // a row of digits: 108, padded to 240 bytes
-constexpr size_t kDigitBytes = (size_t)256 * kRowHalfs * 2;
+// Digits of P, Q in core matrices of 8 rows (k) of 8 columns, 128 bytes; the 14
+// of a row of cores follow each other.
+constexpr int kCores = 14, kCols = 8 * kCores;
+constexpr int kCoreRow = kCores * 128;               // bytes of 8 rows
+constexpr size_t kDigitBytes = 32 * kCoreRow;
 constexpr int kFxUG = kTri * 9 + 4 * 16 * 9;  // int4 of the links and propagators
 constexpr size_t kFxSmem = sizeof(int4) * (kFxUG + 2 * 2304) + 2 * kDigitBytes;
 
 struct FxShared {
   int e[5];                    // largest biased exponents: 4 flavours, links
   int bad;                     // the hypercube does not fit
+  int fail;                    // a wait for the tensor cores ran out
+  unsigned tmem;               // first column of the accumulator
+  unsigned long long done;     // mbarrier: an operator's products are complete
   unsigned long long most[2];  // largest |v| of P and Q before scaling
 };
 
@@ -420,99 +429,100 @@ __device__ __forceinline__ long long fx_scaled(double v, int biased_top) {
   return ((long long)a.h << FX_LOW) + a.l;
 }
 
-// C is kept for the needed blocks only, by rows of digit i: columns 0 ..
-// 18 (7 - i) - 1 (at most 108).
-__device__ __forceinline__ int c_width(int i) { return i == 0 ? 108 : 18 * (7 - i); }
-__device__ __forceinline__ int c_base(int i) {  // of row 18 i
-  return 18 * (i == 0 ? 0 : 108 + 18 * ((i - 1) * 7 - (i * (i - 1)) / 2));
+constexpr int kCRow = 108;                           // floats of a row of C
+static_assert(108 * kCRow * sizeof(float) <= 2 * 2304 * sizeof(longlong2), "C fits where P and Q were");
+constexpr int kTmemCols = 128;
+constexpr unsigned kWaitLimit = 1u << 22;            // polls of an mbarrier: under a second
+constexpr int kIssuer = kFxThreads - 32;             // the thread that issues the products
+
+// byte of (row k, column c) of a digit matrix
+__device__ __forceinline__ unsigned digit_at(int k, int c) {
+  return (k >> 3) * kCoreRow + (c >> 3) * 128 + (k & 7) * 16 + (c & 7) * 2;
 }
 
-constexpr int kCFloats = 18 * (108 + 108 + 90 + 72 + 54 + 36);
-static_assert(2 * kCFloats * sizeof(float) <= 2 * 2304 * sizeof(longlong2), "two C fit where P and Q were");
-
-__device__ __forceinline__ void ldsm4t(unsigned (&r)[4], unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+// Shared-memory descriptor: no swizzle, columns (M, N) contiguous; cores 128
+// bytes apart along the columns, kCoreRow along k.
+__device__ __forceinline__ unsigned long long digit_desc(unsigned addr) {
+  return (unsigned long long)((addr & 0x3ffff) >> 4) | ((unsigned long long)(kCoreRow >> 4) << 16) |
+         ((unsigned long long)(128 >> 4) << 32) | (1ull << 46);
 }
 
-// A warp's tiles of C: m-tile, first n-tile and number of n-tiles (at most 6).
-// Needed n-tiles of the seven m-tiles: 14, 14, 14, 12, 9, 7, 5.
-__device__ __forceinline__ void warp_tiles(int warp, int &mt, int &nt, int &n) {
-  // mt (4 bits), nt (4), n (4) of the 16 warps
-  constexpr unsigned short t[16] = {0x005, 0x055, 0x0a4, 0x105, 0x155, 0x1a4, 0x205, 0x255,
-                                    0x2a4, 0x306, 0x366, 0x405, 0x454, 0x504, 0x543, 0x605};
-  unsigned v = 0;
-#pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (k == warp) v = t[k];
-  mt = v >> 8;
-  nt = (v >> 4) & 15;
-  n = v & 15;
-}
-
-// The digit products of one operator into c (see above) for N n-tiles.
-template <int N>
-__device__ __forceinline__ void digit_tiles(unsigned pd, unsigned qd, NprOp op, float *c, int mt, int nt) {
-  const int lane = threadIdx.x & 31;
-  float acc[N][4];
-#pragma unroll
-  for (int u = 0; u < N; ++u)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[u][e] = 0.f;
-  // the row this lane addresses: matrices (k 0-7, m 0-7), (k 0-7, m 8-15),
-  // (k 8-15, m 0-7), (k 8-15, m 8-15) of A; (k 0-7, n 0-7), (k 8-15, n 0-7),
-  // (k 0-7, n 8-15), (k 8-15, n 8-15) of B
-  const int ka = (lane & 7) + ((lane >> 4) & 1) * 8, kb = (lane & 7) + ((lane >> 3) & 1) * 8;
-  const unsigned a0 = pd + (unsigned)((ka ^ op.t2) * kRowHalfs + mt * 16 + ((lane >> 3) & 1) * 8) * 2;
-  const unsigned b0 = qd + (unsigned)(kb * kRowHalfs + nt * 8 + ((lane >> 4) & 1) * 8) * 2;
-  // signs of the k this lane's fragment registers hold: 2t, 2t + 1 and 8 more
-  const int t2 = 2 * (lane & 3);
-  auto mask = [&](int k) {
-    return (((op.neg2 >> k) & 1u) << 15) | (((op.neg2 >> (k + 1)) & 1u) << 31);
-  };
-  const unsigned lo = mask(t2), hi = mask(t2 + 8);
-#pragma unroll 4
+// C = the digit products of one operator, 128 x 112 x 256, by one thread.
+__device__ __forceinline__ void issue_products(unsigned pd, unsigned qd, int t1, unsigned tmem, unsigned done) {
+  // FP32 sums of FP16 products, both operands contiguous in their columns
+  constexpr unsigned idesc = (1u << 4) | (1u << 15) | (1u << 16) | ((unsigned)(kCols >> 3) << 17) | ((128u >> 4) << 24);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
   for (int A = 0; A < 16; ++A) {
-    const unsigned sa = ((op.neg1 >> A) & 1) ? 0x80008000u : 0u;
-    unsigned a[4], b[(N + 1) / 2][4];
-    ldsm4t(a, a0 + (unsigned)(A * 16 * kRowHalfs * 2));
-    const unsigned ba = b0 + (unsigned)((A ^ op.t1) * 16 * kRowHalfs * 2);
-#pragma unroll
-    for (int u = 0; u < (N + 1) / 2; ++u) ldsm4t(b[u], ba + u * 32);
-    a[0] ^= lo ^ sa;
-    a[1] ^= lo ^ sa;
-    a[2] ^= hi ^ sa;
-    a[3] ^= hi ^ sa;
-#pragma unroll
-    for (int u = 0; u < N; ++u) mma16816(acc[u], a, b[u / 2][2 * (u & 1)], b[u / 2][2 * (u & 1) + 1]);
+    const unsigned long long da = digit_desc(pd + A * 2 * kCoreRow), db = digit_desc(qd + (A ^ t1) * 2 * kCoreRow);
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+        ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(A) : "memory");
   }
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done) : "memory");
+}
+
+__device__ __forceinline__ bool wait_products(unsigned done, unsigned parity) {
+  for (unsigned k = 0; k < kWaitLimit; ++k) {
+    unsigned ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok) : "r"(done), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// The accumulator to C in shared memory: warp w its quarter w % 4 of the rows,
+// 32 columns from 32 (w / 4).
+__device__ __forceinline__ void store_products(unsigned tmem, float *c) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * 32;
+  unsigned v[32];
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(tmem + ((unsigned)((warp & 3) * 32) << 16) + col));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (row < 108) {
 #pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int row = mt * 16 + (lane >> 2) + v * 8, i = row / 18, w = c_width(i);
-    float *cr = c + c_base(i) + (row - 18 * i) * w;
-#pragma unroll
-    for (int u = 0; u < N; ++u) {
-      const int col = (nt + u) * 8 + t2;  // even, as every width is
-      if (row < 108 && col < w) *reinterpret_cast<float2 *>(cr + col) = make_float2(acc[u][2 * v], acc[u][2 * v + 1]);
-    }
+    for (int u = 0; u < 32; u += 4)
+      if (col + u < 108)
+        *reinterpret_cast<uint4 *>(c + row * kCRow + col + u) = make_uint4(v[u], v[u + 1], v[u + 2], v[u + 3]);
   }
 }
 
-// ... by the 16 warps.
-__device__ __forceinline__ void digit_products(unsigned pd, unsigned qd, NprOp op, float *c, int mt, int nt,
-                                               int n) {
-  switch (n) {
-    case 3: digit_tiles<3>(pd, qd, op, c, mt, nt); break;
-    case 4: digit_tiles<4>(pd, qd, op, c, mt, nt); break;
-    case 5: digit_tiles<5>(pd, qd, op, c, mt, nt); break;
-    default: digit_tiles<6>(pd, qd, op, c, mt, nt);
+// Signs and order of C of the digits of Q, from operator `was` (no permutation,
+// no sign if null) to `op`: row (B, c) holds +-Q[B][c ^ t2], of sign
+// neg1[B ^ t1] neg2[c ^ t2], where the rows of P meet it in their own order.
+__device__ __forceinline__ void arrange_q(char *qd, NprOp was, NprOp op) {
+  const int d = was.t2 ^ op.t2;
+  const int bit = d ? 31 - __clz(d) : 3;
+  const int lo = threadIdx.x & 7, B = (threadIdx.x >> 3) & 15;
+  int x = ((lo >> bit) << (bit + 1)) | (lo & ((1 << bit) - 1));
+  // the eight lanes of a 128-byte access on different rows of the two cores
+  if (bit < 3 && (x & 8)) x |= 1 << bit;
+  const int y = d ? x ^ d : x | 8;  // x's partner
+  const unsigned b = ((was.neg1 >> (B ^ was.t1)) ^ (op.neg1 >> (B ^ op.t1))) & 1;
+  auto sign = [&](int c) {  // of the value now at row c, which goes to row c ^ d
+    const unsigned f = b ^ ((was.neg2 >> (c ^ was.t2)) & 1) ^ ((op.neg2 >> (c ^ d ^ op.t2)) & 1);
+    return f ? 0x80008000u : 0u;
+  };
+  const unsigned sx = sign(x), sy = sign(y);
+  for (int n = threadIdx.x >> 7; n < kCores; n += kFxThreads / 128) {
+    uint4 *px = reinterpret_cast<uint4 *>(qd + digit_at(B * 16 + x, n * 8));
+    uint4 *py = reinterpret_cast<uint4 *>(qd + digit_at(B * 16 + y, n * 8));
+    const uint4 vx = *px, vy = *py;
+    *(d ? py : px) = make_uint4(vx.x ^ sx, vx.y ^ sx, vx.z ^ sx, vx.w ^ sx);
+    *(d ? px : py) = make_uint4(vy.x ^ sy, vy.y ^ sy, vy.z ^ sy, vy.w ^ sy);
   }
 }
 
@@ -527,7 +537,7 @@ __device__ __forceinline__ void digit_sum(const float *c, int ra, int rb, long l
 #pragma unroll
     for (int j = 0; j < kDigits; ++j)
       if (i + j <= 6)
-        level[i + j] += __float2int_rn(c[c_base(i) + ra * c_width(i) + 18 * j + rb]);
+        level[i + j] += __float2int_rn(c[(18 * i + ra) * kCRow + 18 * j + rb]);
   hi = ((((long long)level[0] * 512 + level[1]) * 512 + level[2]) * 512) + level[3];
   lo = (((long long)level[4] * 512 + level[5]) * 512) + level[6];
 }
@@ -539,17 +549,27 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
   int4 *gs = ut + kTri * 9;             // [flavour][corner][3][3]
   longlong2 *pq = reinterpret_cast<longlong2 *>(gs + 4 * 16 * 9);  // P [A][D][9], Q [B][C][9]
   float *cm = reinterpret_cast<float *>(pq);                       // C, once these are cut
-  __half *pd = reinterpret_cast<__half *>(pq + 2 * 2304);          // digits of P, then of Q
+  char *pd = reinterpret_cast<char *>(pq + 2 * 2304);              // digits of P, then of Q
   const unsigned pd_s = (unsigned)__cvta_generic_to_shared(pd), qd_s = pd_s + (unsigned)kDigitBytes;
+  const unsigned done = (unsigned)__cvta_generic_to_shared(&sh.done);
   const int tid = threadIdx.x;
   if (tid == 0) {
     for (int k = 0; k < 5; ++k) sh.e[k] = 0;
     sh.bad = 0;
+    sh.fail = 0;
     sh.most[0] = sh.most[1] = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(done) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // columns 108 .. 119 of the digits meet no needed block, but are multiplied
-  for (int i = tid; i < 2 * 256 * (kRowHalfs - 108); i += kFxThreads)
-    pd[(i / (kRowHalfs - 108)) * kRowHalfs + 108 + i % (kRowHalfs - 108)] = __half(0.f);
+  if (tid < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"((unsigned)__cvta_generic_to_shared(&sh.tmem)), "n"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  unsigned phase = 0;
+  // columns 108 .. 111 of the digits meet no output, but are multiplied
+  for (int i = tid; i < 2 * 256; i += kFxThreads)
+    *reinterpret_cast<uint2 *>(pd + (i >> 8) * kDigitBytes + digit_at(i & 255, 108)) = make_uint2(0, 0);
   // this thread's part of an operator's outputs: output o = tid / 4, and the
   // real (0) or imaginary (1) parts of P and Q
   const int o = tid >> 2, part = tid & 3;
@@ -557,8 +577,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
   const int oe = mine ? o : 0;
   const int ra = 2 * (3 * (oe / 27) + oe % 3) + (part >> 1);            // P[a1][a4]
   const int rb = 2 * (3 * ((oe / 3) % 3) + (oe / 9) % 3) + (part & 1);  // Q[a3][a2]
-  int mt, nt, ntiles;
-  warp_tiles(tid >> 5, mt, nt, ntiles);
   double *sum = reinterpret_cast<double *>(a.partial + (long)blockIdx.x * a.nops * 81);
   if (mine && part < 2)
     for (int op = 0; op < a.nops; ++op) sum[2 * (op * 81 + o) + part] = 0.0;
@@ -742,13 +760,13 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
       const unsigned long long re = (unsigned long long)(((v.x + half) >> s) + bias);
       const unsigned long long im = (unsigned long long)(((v.y + half) >> s) + bias);
       const int j = i - k * 2304;
-      __half2 *dst = reinterpret_cast<__half2 *>(pd + k * (256 * kRowHalfs) + (j / 9) * kRowHalfs) + j % 9;
+      char *dst = pd + k * kDigitBytes;
 #pragma unroll
       for (int d = 0; d < kDigits; ++d) {  // from the top
         const int at = kDigitBits * (kDigits - 1 - d);
         const unsigned mr = d ? 511u : 1023u;  // the top field may reach 512
         const unsigned w = ((unsigned)(re >> at) & mr) | (((unsigned)(im >> at) & mr) << 16) | 0x64006400u;
-        dst[9 * d] = __hsub2(*reinterpret_cast<const __half2 *>(&w), __floats2half2_rn(1280.f, 1280.f));
+        *reinterpret_cast<__half2 *>(dst + digit_at(j / 9, 18 * d + 2 * (j % 9))) = __hsub2(*reinterpret_cast<const __half2 *>(&w), __floats2half2_rn(1280.f, 1280.f));
       }
     }
     // units: P 2^(eu + e4 + e1 - vb + s), Q the same with flavours 2, 3; the
@@ -757,28 +775,55 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
     const int ex = 2 * eu + (e[0] + e[1] + e[2] + e[3] - 4 * 1022) + sc[0] + sc[1] - 2 * vb + 7 * kDigitBits;
     const double unit = __hiloint2double((ex + 1023) << 20, 0);
     __syncthreads();
-    // operator op's products while op - 1's are added, C alternating between
-    // two buffers
-#pragma unroll 1
-    for (int op = 0; op <= a.nops; ++op) {
-      if (op < a.nops) digit_products(pd_s, qd_s, a.ops[op], cm + (op & 1) * kCFloats, mt, nt, ntiles);
-      if (op > 0 && tid < 352) {  // whole warps with outputs
-        long long hi, lo;
-        digit_sum(cm + ((op - 1) & 1) * kCFloats, ra, rb, hi, lo);
-        // parts 0..3: re re, re im, im re, im im; part 0 becomes re re - im im,
-        // part 1 re im + im re
-        const long long hx = __shfl_xor_sync(0xffffffffu, hi, 3), lx = __shfl_xor_sync(0xffffffffu, lo, 3);
-        hi += part == 0 ? -hx : hx;
-        lo += part == 0 ? -lx : lx;
-        if (mine && part < 2) {
-          const double d = fma((double)lo, 1.0 / (1 << 27), (double)hi);
-          const int at = (op - 1) * 81 + o;
-          if (a.out_hc) reinterpret_cast<double *>(a.out_hc + (long)h * a.hc_stride + at)[part] = d * unit;
-          sum[2 * at + part] = fma(d, unit, sum[2 * at + part]);
-        }
+    auto add = [&](int op) {  // operator op's outputs from C
+      if (tid >= 352) return;  // whole warps with outputs
+      long long hi, lo;
+      digit_sum(cm, ra, rb, hi, lo);
+      // parts 0..3: re re, re im, im re, im im; part 0 becomes re re - im im,
+      // part 1 re im + im re
+      const long long hx = __shfl_xor_sync(0xffffffffu, hi, 3), lx = __shfl_xor_sync(0xffffffffu, lo, 3);
+      hi += part == 0 ? -hx : hx;
+      lo += part == 0 ? -lx : lx;
+      if (mine && part < 2) {
+        const double d = fma((double)lo, 1.0 / (1 << 27), (double)hi);
+        const int at = op * 81 + o;
+        if (a.out_hc) reinterpret_cast<double *>(a.out_hc + (long)h * a.hc_stride + at)[part] = d * unit;
+        sum[2 * at + part] = fma(d, unit, sum[2 * at + part]);
       }
+    };
+    // operator op's products while op - 1's are added
+    NprOp was = {0, 0, 0, 0};
+#pragma unroll 1
+    for (int op = 0; op < a.nops; ++op) {
+      arrange_q(pd + kDigitBytes, was, a.ops[op]);
+      was = a.ops[op];
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
+      if (tid == kIssuer) issue_products(pd_s, qd_s, was.t1, sh.tmem, done);
+      if (op > 0) add(op - 1);
+      __syncwarp();
+      const bool ok = wait_products(done, phase);
+      phase ^= 1;
+      if (!ok) sh.fail = 1;
+      __syncthreads();
+      if (sh.fail) break;
+      store_products(sh.tmem, cm);
     }
+    if (sh.fail) break;
+    __syncthreads();
+    add(a.nops - 1);
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  if (sh.fail) {  // the same in every thread; loud, and nothing of it is left running
+    wait_products(done, phase ^ 1);
+    if (mine && part < 2)
+      for (int op = 0; op < a.nops; ++op) sum[2 * (op * 81 + o) + part] = __longlong_as_double(-1ll);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (tid < 32) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh.tmem), "n"(kTmemCols));
   }
 }
 

@@ -204,3 +204,19 @@ def test_non_finite_inputs_stay_in_their_hypercube(sq, bad):
     _, hc = _gpu(sq, dims, links, props, OPS16[:3])
     assert not np.isfinite(hc[0]).all()
     _close(hc[1:], want[1:])
+
+
+@pytest.mark.parametrize('seed', [0, 1])
+def test_operators_in_any_order(sq, seed):
+    """Q's digits go from one operator's order and signs to the next one's in
+    place: every change of t1, t2 and the signs between neighbours."""
+    dims = (2, 2, 2, 2)
+    links, props = _inputs(dims)
+    rng = np.random.default_rng(seed)
+    ops = [tuple(int(v) for v in rng.integers(0, 16, 4)) for _ in range(64)]
+    ops += [(0, d, 0, t) for d in range(2) for t in (0, 1, 0, 2, 0, 4, 0, 8, 0, 15, 15, 0, 7)]
+    out, hc = _gpu(sq, dims, links, props, ops)
+    want = oracle.npr_four_fermion(dims, links, props, ops)
+    for k in range(len(ops)):
+        _close(hc[:, k], want[:, k])
+        _close(out[k], want[:, k].sum(axis=0))
