@@ -240,7 +240,7 @@ int sq_spin_taste(int s, int f, int partner[16], int sign[16]);
  * FP64 on the device, for nops operators (S1, F1, S2, F2) (4-bit masks, host
  * array ops[nops][4], 0 <= nops <= 2^20; they are processed SQ_NPR_MAX_OPS at
  * a time, each group recomputing the averaged links and sandwiches -- about
- * a sixth of a group's work at 8 operators, less at 16):
+ * half of a group's time at 8 operators, a third at 16):
  *   O[a1][a2][a3][a4](z) = sum_{A,B,C,D} sum_{c1..c4}
  *       conj(G1(z_A)[c1][a1]) (gamma_S1 x xi_F1)_{AB} G2(z_B)[c2][a2]
  *     * conj(G3(z_C)[c3][a3]) (gamma_S2 x xi_F2)_{CD} G4(z_D)[c4][a4]
@@ -260,7 +260,8 @@ int sq_spin_taste(int s, int f, int partner[16], int sign[16]);
  *               z = z_x + Hx (z_y + Hy (z_z + Hz z_t)), H = L / 2.
  * Device arrays 16-byte aligned; all extents even.  Asynchronous on `stream`,
  * NULL meaning the legacy default stream (a stream-ordered scratch of
- * 16 * 81 * nops bytes per CTA is taken and returned on it).  The sum over z
+ * 16 * 81 * SQ_NPR_MAX_OPS bytes per CTA, and a byte per hypercube, is taken
+ * and returned on it).  The sum over z
  * is deterministic.  The inputs are not checked for finiteness. */
 int npr_four_fermion(sq_ctx *ctx, const int dims[4], const double *links_dev,
                      const double *const props_dev[4], int nops, const int *ops,
@@ -408,8 +409,9 @@ int cg_solve_full(sq_ctx *ctx, int gauge_id, const double *src, double mass, dou
 
 /* out = (m + D) in on the whole lattice, in FP64: the staggered matrix of the
  * paper's inverter (Sec. 2) without even-odd preconditioning.  in_dev/out_dev: distinct device
- * full-lattice vectors [site_lex][colour] complex128.  Uses device scratch
- * for the call (HBM budget) and returns once out is written. */
+ * full-lattice vectors [site_lex][colour] complex128.  Returns once out is
+ * written.  Where the two overlap, or a link's largest element is below 1/16
+ * of the field's, device scratch is used for the call (HBM budget). */
 int dirac_apply(sq_ctx *ctx, int gauge_id, double mass, const double *in_dev, double *out_dev,
                 void *stream);
 

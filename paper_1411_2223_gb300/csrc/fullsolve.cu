@@ -62,16 +62,18 @@ __global__ void __launch_bounds__(128, 4) dirac_fixed_kernel(const __grid_consta
                                                              double mass) {
   griddep_launch_dependents();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.g.vh) return;
-  const SiteCoords sc = site_coords(a.g, a.out_parity, i);
-  const bool active[1] = {true};
-  Vec3<double> acc[1];
-  fixed_hops<1, MODE_PLAIN, IN_FULL>(a, a.ls, sc, i, 0, active, acc);
-  const Vec3<double> v = load_full(a.in, sc.lex);
-  double2 *o = reinterpret_cast<double2 *>(a.out) + (size_t)3 * sc.lex;
+  if (i < a.g.vh) {
+    const SiteCoords sc = site_coords(a.g, a.out_parity, i);
+    const bool active[1] = {true};
+    Vec3<double> acc[1];
+    fixed_hops<1, MODE_PLAIN, IN_FULL>(a, a.ls, sc, i, 0, active, acc);
+    const Vec3<double> v = load_full(a.in, sc.lex);
+    double2 *o = reinterpret_cast<double2 *>(a.out) + (size_t)3 * sc.lex;
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-    o[c] = make_double2(fma(mass, v.c[c].x, 0.5 * acc[0].c[c].x), fma(mass, v.c[c].y, 0.5 * acc[0].c[c].y));
+    for (int c = 0; c < 3; ++c)
+      o[c] = make_double2(fma(mass, v.c[c].x, 0.5 * acc[0].c[c].x), fma(mass, v.c[c].y, 0.5 * acc[0].c[c].y));
+  }
+  griddep_wait();  // the second launch does not end before the first
 }
 
 // out = a x + b y + c z on packed halves of precision P (z may be null)
@@ -396,7 +398,11 @@ extern "C" int dirac_apply(sq_ctx *ctx, int gauge_id, double mass, const double 
   if (!gf->has(PREC_F64, 18)) return SQ_ERR_UNSUPPORTED;
   cudaSetDevice(ctx->device);
   const Geom &g = gf->g;
-  if (gf->fixed) {  // on the caller's own stream
+  // on the caller's own stream; overlapping arrays need the scratch below
+  const size_t n = (size_t)12 * g.vh;  // doubles of a vector
+  const uintptr_t in_b = reinterpret_cast<uintptr_t>(in_dev), out_b = reinterpret_cast<uintptr_t>(out_dev);
+  const bool apart = in_b + n * sizeof(double) <= out_b || out_b + n * sizeof(double) <= in_b;
+  if (gf->fixed && apart) {
     cudaStream_t cs = stream ? (cudaStream_t)stream : cudaStreamLegacy;
     DslashArgs a;
     std::memset(&a, 0, sizeof(a));

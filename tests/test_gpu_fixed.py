@@ -214,3 +214,25 @@ def test_reliable_updates_of_one_system(sq, dims, prec):
             assert abs(st['true_residual'] - true) <= 1e-12
     finally:
         sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('shift', [3, -3])
+def test_dirac_apply_on_overlapping_vectors(sq, shift):
+    """The result is that of separate vectors, as it is written last."""
+    import torch
+    dims = (6, 2, 10, 4)
+    fat, lng = gauge(dims)
+    vol = oracle.volume(dims)
+    v = to_dev(synth.gaussian_source(vol, 9))
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        want = torch.empty_like(v)
+        sq.dirac_apply(gid, 0.07, v, want)
+        both = torch.zeros((vol + abs(shift), 3), dtype=torch.complex128, device='cuda')
+        src, dst = both[max(shift, 0):][:vol], both[max(-shift, 0):][:vol]
+        src.copy_(v)
+        torch.cuda.synchronize()
+        sq.dirac_apply(gid, 0.07, src, dst)
+        assert rel(dst.cpu().numpy(), want.cpu().numpy()) <= 1e-15
+    finally:
+        sq.gauge_free(gid)
