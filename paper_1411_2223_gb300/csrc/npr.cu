@@ -818,6 +818,11 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
     wait_products(done, phase ^ 1);
     if (mine && part < 2)
       for (int op = 0; op < a.nops; ++op) sum[2 * (op * 81 + o) + part] = __longlong_as_double(-1ll);
+    for (; h < a.nhc; h += gridDim.x) {
+      if (tid == 0) a.marked[h] = 0;
+      for (int i = tid; a.out_hc && i < a.nops * 162; i += kFxThreads)
+        reinterpret_cast<double *>(a.out_hc + (long)h * a.hc_stride)[i] = __longlong_as_double(-1ll);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
