@@ -151,11 +151,14 @@ __global__ void __launch_bounds__(128) fatten_kernel(FatGeom g, const double2 *u
 // and every path multiplied out 422.
 //
 // The products run on the integer multiply-add units in the fixed-point form
-// of sq_fixed.cuh when every link's rows and columns have norm 1 to 2^-8, as
-// SU(3) links do.  Every field is then bounded: |U| <= 1, |S| <= 1.02,
-// |A| <= 2.04, |Y| <= 8.2 for Y = the sum in X, as elements and as matrix norms,
-// and |X + c_L S| <= 1.02 (|c3| + 4 |c5| + 8 |c7| + |c_L|) < 2^E, so each is kept
-// at its own fixed unit (55 bits where it is an operand) and no sum overflows:
+// of sq_fixed.cuh when every link is unitary to 2^-9, in each element of
+// U U^dag - 1.  That matrix's norm is then at most 3 sqrt(2) 2^-9, and every
+// field is bounded, as a matrix norm and so in its elements: |U| <= 1.0042,
+// |S| <= 1.013, |A| <= 2.03, |Y| <= 8.17 for Y = the sum in X, and
+// |X + c_L S| <= 1.022 (|c3| + 4 |c5| + 8 |c7| + |c_L|) < 2^E, so each is kept
+// at its own fixed unit (55 bits where it is an operand) and no sum overflows
+// (rows and columns of norm 1 would not do: a 3 x 3 matrix of them can have norm
+// sqrt(3), and Y then passes the 2^58 units that fat_times takes):
 //   U 2^-55, S 2^-55, A 2^-53, Y 2^-55, X 2^(E-60), W = X + c_L S 2^(E-55),
 //   T = U W 2^-1 and S = T U 2^-2 of W's unit, |T| <= 2^57, |S| <= 2^59.6 for six.
 // Other links go through the same kernels in FP64; the flag is on the device
@@ -174,7 +177,7 @@ __global__ void __launch_bounds__(128) fatten_kernel(FatGeom g, const double2 *u
 // (before: 2.8e-16), with only the seven-link paths 7.8e-17 (1.5e-16).
 
 struct FatScale {
-  unsigned uneven;             // a link's row or column norm is not 1
+  unsigned uneven;             // a link is not unitary
 };
 
 // Time slices in scratch: slot (t - t0) mod Lt, slots 0 .. nslots - 1.
@@ -382,22 +385,32 @@ __device__ __forceinline__ void row_staple(const AsqtadArgs &a, const SlabSite &
 // The k-th (0..2) direction besides mu.
 __device__ __forceinline__ int other_dir(int mu, int k) { return k < mu ? k : k + 1; }
 
-// Are the norms of all links' rows and columns 1 to 2^-8?
+// Are all links unitary?  |U U^dag - 1| < 2^-9 in the parts of every element,
+// which NaN and infinities fail.  Bound by the links' loads (295 MB at 20^3 x 64,
+// 44 us of the 8.7 ms).
 __global__ void __launch_bounds__(256) fat_scale_kernel(const double2 *u, long nlinks, FatScale *sc) {
   bool even = true;
   for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nlinks;
        k += (long)gridDim.x * blockDim.x) {
-    float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+    float2 m[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       const double2 v = __ldg(u + k * 9 + e);
-      const float x = (float)v.x, y = (float)v.y, q = fmaf(x, x, y * y);
-      row[e / 3] += q;
-      col[e % 3] += q;
+      m[e] = make_float2((float)v.x, (float)v.y);
     }
 #pragma unroll
-    for (int e = 0; e < 3; ++e)  // false for NaN
-      even = even && fabsf(row[e] - 1.f) < 1.f / 256 && fabsf(col[e] - 1.f) < 1.f / 256;
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j) {
+        float re = i == j ? -1.f : 0.f, im = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float2 x = m[3 * i + c], y = m[3 * j + c];
+          re = fmaf(x.x, y.x, fmaf(x.y, y.y, re));
+          im = fmaf(x.y, y.x, fmaf(-x.x, y.y, im));
+        }
+        even = even && fabsf(re) < 1.f / 512 && fabsf(im) < 1.f / 512;
+      }
   }
   if (!__all_sync(0xffffffffu, even) && (threadIdx.x & 31) == 0) sc->uneven = 1;
 }
@@ -412,7 +425,7 @@ __global__ void __launch_bounds__(128) fat_links_kernel(AsqtadArgs a, const doub
   for (int e = 0; e < 9; ++e) {
     const double2 v = __ldg(thin + (p.lex * 4 + mu) * 9 + e);
     int4 q;
-    if (fixed) {  // |v| <= 1.002: the units of 2^-55 times elements that may reach 2^1
+    if (fixed) {  // |v| <= 1.0042: the units of 2^-55 times elements that may reach 2^1
       const Fx r = fx_from_double(v.x, 1023, 1), i = fx_from_double(v.y, 1023, 1);
       q = fat_word(fat_join(r.l, r.h) * 2, fat_join(i.l, i.h) * 2);
     } else {

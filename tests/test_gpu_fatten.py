@@ -217,3 +217,35 @@ def test_asqtad_non_finite_links(sq, bad):
     assert not np.isfinite(got[0, 0]).all()
     assert np.abs(got[far] - f0[far]).max() <= 1e-14
     assert np.abs(lng.cpu().numpy()[far] - l0[far]).max() <= 1e-15
+
+
+@pytest.mark.parametrize('what', ['ones', 'phases', 'phases_at_random', 'one_link', 'edge', 'past_edge'])
+def test_asqtad_links_with_unit_rows_that_are_not_unitary(sq, what):
+    """Unit rows and columns do not bound a link's matrix norm (all elements
+    1/sqrt(3): norm sqrt(3)), so such links take the FP64 kernels; multiples of
+    unitary links just inside and outside the line between the forms, with
+    constant links, where every staple adds up.  Tolerances as in
+    test_asqtad_forms."""
+    import torch
+    dims = (4, 2, 6, 4)
+    vol = oracle.volume(dims)
+    u = np.empty((vol, 4, 3, 3), dtype=np.complex128)
+    rng = np.random.default_rng(5)
+    if what == 'ones':
+        u[:] = 1 / np.sqrt(3)
+    elif what == 'phases':
+        u[:] = np.array([[1, 1, -1], [1, 1j, 1], [-1j, 1, 1]]) / np.sqrt(3)
+    elif what == 'phases_at_random':
+        u[:] = np.exp(2j * np.pi * rng.uniform(size=u.shape)) / np.sqrt(3)
+    elif what == 'one_link':
+        u[:] = synth.thin_links(dims, 0.7, 3)
+        u[vol // 2, 1] = 1 / np.sqrt(3)
+    else:
+        u[:] = np.eye(3) * np.sqrt(1 + (0.9 if what == 'edge' else 1.1) / 512)
+    t = torch.from_numpy(u).cuda()
+    fat, lng = torch.full_like(t, float('nan')), torch.full_like(t, float('nan'))
+    sq.gauge_fatten_asqtad(dims, t, fat, lng)
+    f0, l0 = _asqtad_ref(dims, u, sq.ASQTAD_COEFFS)
+    for got, want in ((fat.cpu().numpy(), f0), (lng.cpu().numpy(), l0)):
+        assert rel(got, want) <= 2e-15
+        assert np.abs(got - want).max() <= 1e-14 * np.abs(want).max()
