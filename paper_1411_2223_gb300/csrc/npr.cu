@@ -38,8 +38,10 @@
 //     exactly, and the digits' products are summed over the 256 (A, C) by
 //     tcgen05.mma into FP32 accumulators in TMEM, exactly (256 256 256 = 2^24).
 // A hypercube whose inputs or averaged links do not fit that form (infinities,
-// NaN, elements near the ends of FP64, links far from unitary) is marked there
-// and computed by npr_fp64_kernel in FP64.
+// NaN, elements near the ends of FP64, links far from unitary), or of which an
+// output is so much smaller than the largest products of its P and Q that the
+// form's one scale would cost it digits (kRough below), is marked there and
+// computed by npr_fp64_kernel in FP64.
 // Per-hypercube results are written when asked for; the sums over hypercubes
 // go through per-CTA partials and a fixed-order second pass, so they do not
 // depend on scheduling.
@@ -354,6 +356,24 @@ __global__ void __launch_bounds__(kThreads, 1) npr_fp64_kernel(const NprArgs a) 
 // operator: reordering Q, and C from TMEM through shared memory.  Error of a
 // hypercube against long double 3.2e-16 to 3.6e-16, with FP64 FMAs (three per
 // complex term) 4.6e-16.
+//
+// One scale for all of P and Q: an output is a sum of P[A][D] Q[C][B] over
+// pairs of corners that the operator picks, and where the flavours peak at
+// different corners (or source colours) it has only products of large P with
+// small Q and the other way round, while P and Q are rounded to 2^-54 of their
+// largest elements.  With g_f(c, a) the norm of flavour f's column a at corner c,
+// an output's FP64 rounding goes with R, its rounding here with M,
+//   R^2 = sum_A g1(A, a1)^2 g2(A ^ t1, a2)^2  sum_C g3(C, a3)^2 g4(C ^ t2, a4)^2,
+//   M^2 = |P|max^2 sum g3^2 sum g2^2 + |Q|max^2 sum g1^2 sum g4^2.
+// A hypercube with M > 12 R in any output and for any t1, t2 (so that it does not
+// depend on the other operators of the call) goes to npr_fp64_kernel.  The
+// largest error of a hypercube's outputs, each over the root of the sum of its
+// |P|^2 |Q|^2, is 0.9e-15 at M / R = 5, 1.1e-15 at 7, 1.6e-15 at 12, 2.3e-15 at 20
+// and 1e-14 at 100, and 1.7e-15 with FP64 FMAs (medians, the steps in long
+// double).  Gaussian propagators have M / R of 5, above 8 in 1 % of the
+// hypercubes and above 11 in none of 20000; with peaks of 2 at opposite corners
+// it is 9 to 16, of 8 200 to 400.  The norms and the comparison cost 2.6 % of the
+// call (16^3 x 32, 8 operators: 2.11 to 2.165 ms).
 struct FxC { Fx re, im; };
 struct Wide { long long hr, mr, hi, mi; };
 
@@ -403,6 +423,7 @@ constexpr long long kFxMost = 1ll << (FX_LOW + 30);  // two words hold values be
 constexpr int kPropBits = FX_BITS, kLinkBits = 56;   // bits at the blocks' scales
 constexpr int kMidBits = 55;                         // ... of U G4 and U G2
 constexpr int kDigits = 6, kDigitBits = 9;
+constexpr float kRough = 144.f;                      // largest M^2 / R^2 of an output
 constexpr int kPQBits = kDigits * kDigitBits - 1;    // P and Q: |v| <= 2^53
 // Digits of P, Q in core matrices of 8 rows (k) of 8 columns, 128 bytes; the 14
 // of a row of cores follow each other.
@@ -419,6 +440,10 @@ struct FxShared {
   unsigned tmem;               // first column of the accumulator
   unsigned long long done;     // mbarrier: an operator's products are complete
   unsigned long long most[2];  // largest |v| of P and Q before scaling
+  unsigned seen;               // bit 3 f + a: column a of flavour f has a nonzero element
+  float g2[4][16][3];          // squared norms of the propagators' columns, at the scales
+  float g2_sum[4][3];          // ... summed over the corners
+  float pair[18];              // the sums of R^2: least over t1 of 3 a1 + a2, then over t2 of 3 a3 + a4
 };
 
 __device__ __forceinline__ int fx_biased(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
@@ -557,6 +582,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
     for (int k = 0; k < 5; ++k) sh.e[k] = 0;
     sh.bad = 0;
     sh.fail = 0;
+    sh.seen = 0;
     sh.most[0] = sh.most[1] = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(done) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -620,6 +646,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
       if (e[k] == 0) e[k] = 1022;  // all zero (or denormal: see below)
       else fits &= k == 4 ? (e[k] >= 1022 - 1 && e[k] <= 1022 + 2) : (e[k] >= 1022 - 200 && e[k] <= 1022 + 200);
     }
+    unsigned seen = 0;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int i = tid + k * kFxThreads;
@@ -632,7 +659,10 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
       *own[k] = fx_word(fx_scaled(raw[k].x, top) << up, fx_scaled(raw[k].y, top) << up);
       if (fx_biased(raw[k].x) == 0) fits &= raw[k].x == 0.0;  // no denormals
       if (fx_biased(raw[k].y) == 0) fits &= raw[k].y == 0.0;
+      if (i < 576 && (raw[k].x != 0.0 || raw[k].y != 0.0)) seen |= 1u << (3 * (i / 144) + i % 3);
     }
+    seen = __reduce_or_sync(0xffffffffu, seen);
+    if ((tid & 31) == 0) atomicOr(&sh.seen, seen);
     const int eu = e[4] - 1022;  // |link element| < 2^eu
     const int one = min(kLinkBits - eu, kLinkBits + 1);  // U_AA = 1 in the links' units
     if (tid < 144) {
@@ -678,6 +708,32 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
         // the elements' bound: 2^eu, as for unitary links
         if (max(abs64(re), abs64(im)) > 1ll << kLinkBits) sh.bad = 1;
         ut[tri(A, D) * 9 + el] = fx_word(re, im);
+      } else if (n == 3 && tid >= 320) {  // threads without a pair: M and R's norms
+        const int k = tid - 320;
+        const int4 *g = gs + (k / 3) * 9 + k % 3;
+        float q = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int4 v = g[3 * c];
+          const float re = fmaf((float)v.y, 0x1p-28f, (float)v.x * 0x1p-55f);
+          const float im = fmaf((float)v.w, 0x1p-28f, (float)v.z * 0x1p-55f);
+          q = fmaf(re, re, fmaf(im, im, q));
+        }
+        sh.g2[k / 48][(k / 3) % 16][k % 3] = q;
+      } else if (n == 4 && tid >= 96 && tid < 384) {  // t in the 16 lanes, the sum's columns
+        const int k = (tid - 96) >> 4, t = tid & 15;
+        const int f = k < 9 ? 0 : 2, a = (k % 9) / 3, b = k % 3;
+        float q = 0.f;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) q = fmaf(sh.g2[f][c][a], sh.g2[f + 1][c ^ t][b], q);
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) q = fminf(q, __shfl_xor_sync(0xffffffffu, q, d));
+        if (t == 0) sh.pair[k] = q;
+      } else if (n == 4 && tid >= 384 && tid < 396) {
+        const int f = (tid - 384) / 3, a = tid % 3;
+        float q = 0.f;
+        for (int c = 0; c < 16; ++c) q += sh.g2[f][c][a];
+        sh.g2_sum[f][a] = q;
       }
       __syncthreads();
     }
@@ -731,15 +787,27 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
     }
     if (big) sh.bad = 1;
     __syncthreads();
-    const bool bad = sh.bad != 0;
+    constexpr int vb = kMidBits + kPropBits - 2 * FX_LOW + 2;  // bits of |v| at scale 1
     // P and Q at their own scales
     int sc[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) sc[k] = max(0, 64 - __clzll((long long)sh.most[k]) - kPQBits);
-    __syncthreads();
+    bool rough = false;  // output tid: M^2 > kRough R^2, of columns that are not all zero
+    if (tid < 81) {
+      const int a1 = tid / 27, a2 = (tid / 9) % 3, a3 = (tid / 3) % 3, a4 = tid % 3;
+      // |P|max, |Q|max as powers of two; the steps before P and Q round to the
+      // propagators' scales, which counts as 1/2 of their product
+      const float p = __int_as_float((max(sc[0] + kPQBits + eu - vb, -1) + 127) << 23);
+      const float q = __int_as_float((max(sc[1] + kPQBits + eu - vb, -1) + 127) << 23);
+      const float m2 = fmaf(p * p, sh.g2_sum[2][a3] * sh.g2_sum[1][a2], q * q * (sh.g2_sum[0][a1] * sh.g2_sum[3][a4]));
+      const unsigned cols = 1u << a1 | 8u << a2 | 64u << a3 | 512u << a4;
+      rough = (sh.seen & cols) == cols && !(m2 <= kRough * sh.pair[3 * a1 + a2] * sh.pair[9 + 3 * a3 + a4]);
+    }
+    const bool bad = __syncthreads_or(rough || sh.bad != 0);
     if (tid == 0) {
       for (int k = 0; k < 5; ++k) sh.e[k] = 0;
       sh.bad = 0;
+      sh.seen = 0;
       sh.most[0] = sh.most[1] = 0;
       a.marked[h] = bad;
       if (bad) *a.any_marked = 1;
@@ -771,7 +839,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
     }
     // units: P 2^(eu + e4 + e1 - vb + s), Q the same with flavours 2, 3; the
     // sums are in 512^7 of their product
-    constexpr int vb = kMidBits + kPropBits - 2 * FX_LOW + 2;  // bits of |v| at scale 1
     const int ex = 2 * eu + (e[0] + e[1] + e[2] + e[3] - 4 * 1022) + sc[0] + sc[1] - 2 * vb + 7 * kDigitBits;
     const double unit = __hiloint2double((ex + 1023) << 20, 0);
     __syncthreads();

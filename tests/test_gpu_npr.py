@@ -220,3 +220,80 @@ def test_operators_in_any_order(sq, seed):
     for k in range(len(ops)):
         _close(hc[:, k], want[:, k])
         _close(out[k], want[:, k].sum(axis=0))
+
+
+def _averaged_links(dims, links):
+    """U[hypercube][A][D], the means over the shortest paths, in long double."""
+    lx, ly, lz, lt = dims
+    z = np.indices([d // 2 for d in dims][::-1]).reshape(4, -1)[::-1]
+    st = np.array([1, lx, lx * ly, lx * ly * lz])
+    base = 2 * (z * st[:, None]).sum(0)
+    site = np.stack([base + sum(st[m] for m in range(4) if a >> m & 1) for a in range(16)], 1)
+    u = np.zeros((len(base), 16, 16, 3, 3), dtype=np.clongdouble)
+    u[:, range(16), range(16)] = np.eye(3)
+    l = links.astype(np.clongdouble)
+    for n in range(1, 5):
+        for a in range(16):
+            for x in (x for x in range(16) if bin(x).count('1') == n):
+                for m in (m for m in range(4) if x >> m & 1):
+                    b = a ^ (1 << m)
+                    s = l[site[:, a], m] if b > a else np.conj(np.swapaxes(l[site[:, b], m], 1, 2))
+                    u[:, a, a ^ x] += s @ u[:, b, a ^ x] / np.longdouble(n)
+    return site, u
+
+
+def _sandwiches(dims, links, props):
+    site, u = _averaged_links(dims, links)
+    g = [p.astype(np.clongdouble)[site] for p in props]
+    p = np.einsum('hxca,hxycd,hydb->hxyab', np.conj(g[0]), u, g[3], optimize=True)
+    q = np.einsum('hxca,hxycd,hydb->hxyab', np.conj(g[2]), u, g[1], optimize=True)
+    return p, q
+
+
+@pytest.mark.parametrize('what', ['gauss', 'opposite2', 'opposite8', 'opposite64', 'opposite1024',
+                                  'corners', 'columns', 'disjoint', 'zero_corner', 'tiny_column',
+                                  'one_column'])
+def test_every_output_on_the_scale_of_its_own_products(sq, what):
+    """Flavours that peak at different corners or source colours.  An output
+    sums 256 products of P and Q: with R the root of the sum of their squared
+    magnitudes, FP64 rounding leaves some 2e-15 R at most (P and Q a few ulp
+    each, sums of 64 terms); 64 ulp of R = 7.1e-15 is allowed, against long
+    double."""
+    dims = (4, 4, 2, 4)
+    links, props = _inputs(dims, seed=8)
+    vol = oracle.volume(dims)
+    rng = np.random.default_rng(9)
+    lx, ly, lz, lt = dims
+    lex = np.arange(vol)
+    corner = (lex % lx & 1) + 2 * (lex // lx % ly & 1) + 4 * (lex // (lx * ly) % lz & 1) + \
+        8 * (lex // (lx * ly * lz) & 1)
+    s = [np.ones((vol, 1, 3)) for _ in range(4)]
+    if what.startswith('opposite'):
+        for f, c in ((0, 0), (3, 0), (1, 15), (2, 15)):
+            s[f][corner == c] = float(what[8:])
+    elif what == 'corners':
+        s = [np.exp(rng.uniform(-3, 3, (vol, 1, 1))) * np.ones((1, 1, 3)) for _ in range(4)]
+    elif what == 'columns':
+        s = [np.exp(rng.uniform(-2, 2, (1, 1, 3))) * np.ones((vol, 1, 1)) for _ in range(4)]
+    elif what == 'disjoint':  # no operator has all its products zero, most have few
+        for f, c in ((0, 3), (1, 3), (2, 5), (3, 6)):
+            s[f][(corner & c) != 0] = 0.0
+    elif what == 'zero_corner':
+        s[1][corner == 6] = 0.0
+    elif what == 'tiny_column':
+        s[2][:, :, 1] = 1e-20
+    elif what == 'one_column':
+        for f in range(4):
+            s[f][:, :, 1:] = 0.0
+    props = [p * w for p, w in zip(props, s)]
+    ops = OPS16[:4] + OPS16[8:]
+    _, hc = _gpu(sq, dims, links, props, ops)
+    p, q = _sandwiches(dims, links, props)
+    a = np.arange(16)
+    for k, (s1, f1, s2, f2) in enumerate(ops):
+        sign = [oracle.spin_taste(x, y)[a, a ^ x ^ y].real for x, y in ((s1, f1), (s2, f2))]
+        pk = p[:, :, a ^ s2 ^ f2] * (sign[0][:, None] * sign[1][None, :])[None, :, :, None, None]
+        qk = q[:, :, a ^ s1 ^ f1].transpose(0, 2, 1, 3, 4)  # [A][C]
+        want = np.einsum('hacxw,haczy->hxyzw', pk, qk)
+        r = np.sqrt(np.einsum('hacxw,haczy->hxyzw', np.abs(pk) ** 2, np.abs(qk) ** 2))
+        assert np.all(np.abs(hc[:, k] - want) <= 64 * 2.0 ** -53 * r)
