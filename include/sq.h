@@ -410,8 +410,9 @@ int cg_solve_full(sq_ctx *ctx, int gauge_id, const double *src, double mass, dou
 /* out = (m + D) in on the whole lattice, in FP64: the staggered matrix of the
  * paper's inverter (Sec. 2) without even-odd preconditioning.  in_dev/out_dev: distinct device
  * full-lattice vectors [site_lex][colour] complex128.  Returns once out is
- * written.  Where the two overlap, or a link's largest element is below 1/16
- * of the field's, device scratch is used for the call (HBM budget). */
+ * written.  Where the two overlap, or where a fat link's largest element is
+ * below a 16th to 32nd of the field's or a long link's below a 256th to 512th
+ * (long links of zero apart), device scratch is used for the call (HBM budget). */
 int dirac_apply(sq_ctx *ctx, int gauge_id, double mass, const double *in_dev, double *out_dev,
                 void *stream);
 

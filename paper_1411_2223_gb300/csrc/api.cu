@@ -276,7 +276,7 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
     if (std::abs(det.imag()) > 1e-10 * std::abs(det) || gf->long_s == 0) gf->long_s = 0;
   }
   unsigned long long *stats_d = nullptr;
-  unsigned long long stats_h[4] = {0, 0, 0, 0};
+  unsigned long long stats_h[5] = {0, 0, 0, 0, 0};
   cudaError_t e = cudaMalloc(&stats_d, sizeof(stats_h));
   if (e == cudaSuccess) {
     cudaMemsetAsync(stats_d, 0, sizeof(stats_h), st);
@@ -291,12 +291,13 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
     if (tmp) cudaFree(tmp);
     return SQ_ERR_CUDA;
   }
-  double fmax_, lmax_, rerr, least;
+  double fmax_, lmax_, rerr, fleast, lleast;
   std::memcpy(&fmax_, &stats_h[0], 8);
   std::memcpy(&lmax_, &stats_h[1], 8);
   std::memcpy(&rerr, &stats_h[2], 8);
-  stats_h[3] = ~stats_h[3];
-  std::memcpy(&least, &stats_h[3], 8);
+  for (int k = 3; k < 5; ++k) stats_h[k] = ~stats_h[k];
+  std::memcpy(&fleast, &stats_h[3], 8);
+  std::memcpy(&lleast, &stats_h[4], 8);
   if (!std::isfinite(fmax_) || !std::isfinite(lmax_)) {
     if (tmp) cudaFree(tmp);
     return SQ_ERR_NONFINITE;
@@ -304,13 +305,15 @@ extern "C" int gauge_load(sq_ctx *ctx, const int dims[4], const double *fat, con
   gf->fat_scale = (float)fmax_;
   gf->long_scale = (float)lmax_;
   gf->recon12_ok = gf->long_s != 0 && rerr <= 1e-10 * std::abs(gf->long_s);
-  // Fixed-point FP64 links hold every element to 2^-56 of the field's largest:
-  // finer than FP64's own rounding of the mat-vecs while each direction's
-  // links reach 2^-4 of that largest element.  Fields with smaller links (or
-  // elements that are not finite) keep doubles and FP64 FMAs.
+  // Fixed-point FP64 links hold every fat element to 2^-56 of the field's largest
+  // and every long one to 2^-61: about FP64's rounding of a link of the least size
+  // that is taken.  Fields with smaller links (long links of zero apart) or with
+  // elements that are not finite keep doubles and FP64 FMAs.
   const double lmost = std::max(fmax_, lmax_);
   if (lmost > 0) gf->fixed_exp = std::ilogb(lmost) + 1;
-  gf->fixed = lmost > 0 && least >= lmost / 16 && std::abs(gf->fixed_exp) <= 60;
+  gf->fixed = lmost > 0 && std::abs(gf->fixed_exp) <= 60 &&
+              fleast >= std::ldexp(1.0, gf->fixed_exp - FX_FAT_LEAST) &&
+              lleast >= std::ldexp(1.0, gf->fixed_exp - FX_LONG_LEAST);
   PackScales ps;
   ps.to_fixed = gf->fixed ? std::ldexp(1.0, FX_BITS - gf->fixed_exp) : 0.0;
   ps.fat_inv = gf->fat_scale > 0 ? 32767.0f / gf->fat_scale : 0.f;

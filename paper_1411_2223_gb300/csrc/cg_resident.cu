@@ -128,11 +128,11 @@ __device__ __forceinline__ Vec3<R> split_dslash(const DslashArgs &a, bool valid,
   const bool active[1] = {true};
   Vec3<R> acc[1];
   zero(acc[0]);
-  bool odd = false;
+  FxForm form = {0, 0, false};
   if (valid) {
     const SiteCoords sc = site_coords(g, a.out_parity, i);
     if constexpr (PREC == PREC_F64) {
-      fixed_hops<1, MODE_PLAIN, IN_CO>(a, a.ls, sc, i, 0, active, acc, sub, SPLIT, &odd);
+      fixed_hops<1, MODE_PLAIN, IN_CO>(a, a.ls, sc, i, 0, active, acc, sub, SPLIT, &form);
     } else {
 #pragma unroll 1
       for (int mu = sub; mu < 4; mu += SPLIT) {
@@ -170,6 +170,23 @@ __device__ __forceinline__ Vec3<R> split_dslash(const DslashArgs &a, bool valid,
       }
     }
   }
+  if constexpr (PREC == PREC_F64) {
+    // of all directions: the exponents' maxima and whether a neighbour was odd
+    const bool odd_here = form.odd;
+#pragma unroll
+    for (int d = 1; d < SPLIT; d <<= 1) {
+      form.e = max(form.e, __shfl_xor_sync(0xffffffffu, form.e, d));
+      form.fat = max(form.fat, __shfl_xor_sync(0xffffffffu, form.fat, d));
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, odd_here);
+    form.odd = (who & (((1u << SPLIT) - 1) << ((threadIdx.x & 31) / SPLIT * SPLIT))) != 0;
+    if (!form.odd && form.apart()) {  // each lane its directions, as before
+      double o[6];
+      fixed_site_apart<IN_CO>(a, i, 0, form, sub, SPLIT, o);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[0].c[c] = make_double2(o[2 * c], o[2 * c + 1]);
+    }
+  }
 #pragma unroll
   for (int d = 1; d < SPLIT; d <<= 1)
 #pragma unroll
@@ -178,9 +195,7 @@ __device__ __forceinline__ Vec3<R> split_dslash(const DslashArgs &a, bool valid,
       acc[0].c[c].y += __shfl_xor_sync(0xffffffffu, acc[0].c[c].y, d);
     }
   if constexpr (PREC == PREC_F64) {
-    const unsigned who = __ballot_sync(0xffffffffu, odd);
-    const unsigned mine = ((1u << SPLIT) - 1) << ((threadIdx.x & 31) / SPLIT * SPLIT);
-    if (who & mine) {
+    if (form.odd) {
       double o[6];
       fixed_site_fp64<MODE_PLAIN, IN_CO>(a, i, 0, o);
 #pragma unroll

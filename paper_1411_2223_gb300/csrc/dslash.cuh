@@ -332,7 +332,13 @@ __device__ __forceinline__ void pair_hops(const DslashArgs &a, const LinkScales 
 // flight (168 registers, three blocks) was slower: 113 against 110 us for one
 // system at 20^3 x 64, 1120 against 999 us for 12.  Neighbours outside the fixed-point range
 // (infinities, NaN, magnitudes near the ends of FP64) send the site to
-// fixed_site_fp64.
+// fixed_site_fp64, neighbours that are much smaller by the fat hops than by the long
+// ones (FX_KINDS_APART) to fixed_site_apart.
+// Keeping the digits of such sites in the sums instead was slower: 14 x 18 x 22 x
+// 54, one and 12 systems 66 and 611 us; with the long links at a unit of their own
+// and all long hops before the fat ones, the sums shifted between, 73 and 701 us
+// (the hops of a direction no longer meet in L1); with each long row summed apart
+// and added, 78 and 736 us.
 
 // Input of the FP64 operators: packed half vectors, the reliable update's
 // x64 + xs, or a canonical whole-lattice vector [site_lex][colour].
@@ -401,8 +407,12 @@ __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs
 #pragma unroll 1
     for (int e = 0; e < 9; ++e) {
       const int4 q = m[(size_t)e * S];
-      const double mr = ((double)q.y * (1 << FX_LOW) + (double)q.x) * unit;
-      const double mi = ((double)q.w * (1 << FX_LOW) + (double)q.z) * unit;
+      // of a long link, in units of 2^-FX_MORE and with half of them added
+      const double up = h & 2 ? 1ll << (FX_LOW + FX_MORE) : 1 << FX_LOW;
+      const double off = h & 2 ? 1 << (FX_MORE - 1) : 0;
+      const double ue = h & 2 ? unit / (1 << FX_MORE) : unit;
+      const double mr = fma((double)q.y, up, (double)q.x - off) * ue;
+      const double mi = fma((double)q.w, up, (double)q.z - off) * ue;
       const int r = e / 3, c = e % 3;
       const double2 w = c == 0 ? v.c[0] : c == 1 ? v.c[1] : v.c[2];
       acc[2 * r] = fma(mr, w.x, fma(-mi, w.y, acc[2 * r]));
@@ -413,31 +423,118 @@ __device__ __noinline__ void fixed_site_fp64(const DslashArgs &a, int i, int rhs
   for (int c = 0; c < 6; ++c) out[c] = acc[c];
 }
 
-// Directions mu0, mu0 + step, ...; with step > 1 `odd_site` says that a
-// neighbour was outside the range, and the caller has the site recomputed.
+// What the hops of a site say about its form.
+struct FxForm {
+  int e, fat;  // exponent of the sums, and of the largest fat-hop neighbour
+  bool odd;    // a neighbour outside the fixed-point range: fixed_site_fp64
+  __device__ __forceinline__ bool apart() const {  // fixed_site_apart
+    return e > FX_MIN_E && fat < e - 1 - FX_KINDS_APART;
+  }
+};
+
+// The fat hops and the long hops apart, each relative to an exponent of its own
+// neighbours, every product whole and the long links' further bits among them;
+// one rounding more, where the two results are added.  Directions mu0, mu0 +
+// step, ...; one hop's code, as few sites come here.
+template <int IN>
+__device__ __noinline__ void fixed_site_apart(const DslashArgs &a, int i, int rhs, const FxForm fm,
+                                              int mu0, int step, double *out) {
+  const Geom &g = a.g;
+  const int S = g.stride;
+  const SiteCoords sc = site_coords(g, a.out_parity, i);
+#pragma unroll 1
+  for (int lng = 0; lng < 2; ++lng) {
+    const int E = lng ? fm.e : max(fm.fat + 1, FX_MIN_E);
+    FxAcc s;
+    fx_zero(s);
+    long long lr[3] = {0, 0, 0}, li[3] = {0, 0, 0};  // products of low words
+#pragma unroll 1
+    for (int k = 2 * mu0; k < 8; k += (k & 1) ? 2 * step - 1 : 1) {
+      const int mu = k >> 1, back = k & 1;
+      float f;
+      int n = hop_index(g, sc, mu, (lng ? 3 : 1) * (back ? -1 : 1), f);
+      const int sgn = f * eta_sign(sc, mu) * (back ? -1.f : 1.f) < 0.f ? -1 : 1;
+      if constexpr (IN == IN_FULL) n = site_coords(g, 1 - a.out_parity, n).lex;
+      Vec3<double> v, d;
+      fx_gather<IN>(a, rhs, S, n, v, d);
+      const int4 *m = reinterpret_cast<const int4 *>(a.links) + (size_t)(4 * mu + 2 * lng + back) * 9 * S + i;
+      int4 q[9];
+#pragma unroll
+      for (int e = 0; e < 9; ++e) q[e] = __ldg(m + (size_t)e * S);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        Fx wr, wi;
+        fx_colour<IN == IN_XS>(v, d, E, sgn, c, wr, wi);
+        const Fx ni = {-wi.h, -wi.l};
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          const int4 t = q[3 * r + c], u = lng ? fx_long_element(t) : t;
+          const int xr = lng ? fx_long_rest(t.x) : 0, xi = lng ? fx_long_rest(t.z) : 0;
+          const Fx mr = {u.y, u.x}, mi = {u.w, u.z};
+          fx_mac(s.hr[r], s.mr[r], mr, wr);
+          fx_mac(s.hi[r], s.mi[r], mr, wi);
+          fx_mac(s.hr[r], s.mr[r], mi, ni);
+          fx_mac(s.hi[r], s.mi[r], mi, wr);
+          fx_mac1(lr[r], mr.l, wr.l);
+          fx_mac1(lr[r], mi.l, ni.l);
+          fx_mac1(li[r], mr.l, wi.l);
+          fx_mac1(li[r], mi.l, wr.l);
+          lr[r] += ((long long)xr * wr.h + (long long)xi * ni.h) * (1 << (FX_LOW - FX_MORE));
+          li[r] += ((long long)xr * wi.h + (long long)xi * wr.h) * (1 << (FX_LOW - FX_MORE));
+        }
+      }
+    }
+    const double unit = fx_unit(a.ls.fixed_exp, E);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double re = fx_to_double(s.hr[c], s.mr[c] + (lr[c] >> FX_LOW), unit);
+      const double im = fx_to_double(s.hi[c], s.mi[c] + (li[c] >> FX_LOW), unit);
+      out[2 * c] = lng ? out[2 * c] + re : re;
+      out[2 * c + 1] = lng ? out[2 * c + 1] + im : im;
+    }
+  }
+}
+
+// One of the two other forms where the site needs it.
+template <int MODE, int IN>
+__device__ __forceinline__ void fixed_site_again(const FxForm &fm, const DslashArgs &a, int i, int rhs,
+                                                 Vec3<double> &acc) {
+  if (!fm.odd && !fm.apart()) return;
+  double o[6];
+  if (fm.odd) fixed_site_fp64<MODE, IN>(a, i, rhs, o);
+  else fixed_site_apart<IN>(a, i, rhs, fm, 0, 1, o);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) acc.c[c] = make_double2(o[2 * c], o[2 * c + 1]);
+}
+
+// Directions mu0, mu0 + step, ...; with step > 1 the caller puts the directions'
+// forms (`form`) together and has the site recomputed where it needs FP64.
 template <int NR, int MODE, int IN>
 __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales &ls,
                                            const SiteCoords &sc, int i, int r0,
                                            const bool (&active)[NR], Vec3<double> (&acc)[NR],
-                                           int mu0 = 0, int step = 1, bool *odd_site = nullptr) {
+                                           int mu0 = 0, int step = 1, FxForm *form = nullptr) {
   constexpr bool XS = IN == IN_XS;
   const Geom &g = a.g;
   const int S = g.stride;
   const uint64_t pol = l2_link_policy(ls.keep, ls.share);
   FxAcc s[NR];
   bool odd[NR];  // a neighbour outside the fixed-point range
+  int fat[NR];   // largest exponent by the fat hops
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
     fx_zero(s[r]);
     odd[r] = false;
+    fat[r] = 0;
   }
-  auto one = [&](int k, int nb, float f) {
+  auto one = [&](int k, bool lng, int nb, float f) {
     int4 m[9];
     const char *base = a.links + ((size_t)k * 9 * S + i) * 16;
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       const uint4 q = ld_stream_u4(base + (size_t)e * S * 16, pol);
       m[e] = make_int4((int)q.x, (int)q.y, (int)q.z, (int)q.w);
+      if (lng) m[e] = fx_long_element(m[e]);
     }
     const int sgn = f < 0.f ? -1 : 1;
 #pragma unroll
@@ -447,6 +544,7 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
       fx_gather<IN>(a, r0 + r, S, nb, v, d);
       int e = fx_max_exponent(v);
       if (XS) e = max(e, fx_max_exponent(d));
+      if (!lng) fat[r] = max(fat[r], e);
       if (e >= s[r].E) {
         if (e >= FX_MAX_E) {
           odd[r] = true;
@@ -459,21 +557,7 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
       }
       FxVec w;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        w.re[c] = fx_from_double(v.c[c].x, s[r].E, sgn);
-        w.im[c] = fx_from_double(v.c[c].y, s[r].E, sgn);
-      }
-      if (XS) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const Fx p = fx_from_double(d.c[c].x, s[r].E, sgn), q = fx_from_double(d.c[c].y, s[r].E, sgn);
-          const int lr = w.re[c].l + p.l, li = w.im[c].l + q.l;
-          w.re[c].h += p.h + (lr >> FX_LOW);
-          w.re[c].l = lr & FX_LOW_MASK;
-          w.im[c].h += q.h + (li >> FX_LOW);
-          w.im[c].l = li & FX_LOW_MASK;
-        }
-      }
+      for (int c = 0; c < 3; ++c) fx_colour<XS>(v, d, s[r].E, sgn, c, w.re[c], w.im[c]);
       fx_mat_vec(s[r], m, w);
     }
   };
@@ -483,33 +567,25 @@ __device__ __forceinline__ void fixed_hops(const DslashArgs &a, const LinkScales
     auto to = [](int lex) { return IN == IN_FULL ? lex : lex >> 1; };
     float f;
     int n = to(hop_lex<+1>(g, sc, mu, f));
-    one(4 * mu, n, eta * f);
+    one(4 * mu, false, n, eta * f);
     n = to(hop_lex<-1>(g, sc, mu, f));
-    one(4 * mu + 1, n, -eta * f);
+    one(4 * mu + 1, false, n, -eta * f);
     n = to(hop_lex<+3>(g, sc, mu, f));
-    one(4 * mu + 2, n, eta * f);
+    one(4 * mu + 2, true, n, eta * f);
     n = to(hop_lex<-3>(g, sc, mu, f));
-    one(4 * mu + 3, n, -eta * f);
+    one(4 * mu + 3, true, n, -eta * f);
   }
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    // products are in units of 2^(fixed_exp - FX_BITS) 2^(E - 1022 - FX_BITS),
-    // the sums of 2^(2 FX_LOW) of these
-    const int ex = ls.fixed_exp + s[r].E - 1022 - 2 * FX_BITS + 2 * FX_LOW;
-    const double unit = __hiloint2double((ex + 1023) << 20, 0);
+    const double unit = fx_unit(ls.fixed_exp, s[r].E);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       acc[r].c[c].x = fx_to_double(s[r].hr[c], s[r].mr[c], unit);
       acc[r].c[c].y = fx_to_double(s[r].hi[c], s[r].mi[c], unit);
     }
-    if (odd_site != nullptr) {
-      *odd_site = odd[r];
-    } else if (active[r] && odd[r]) {
-      double o[6];
-      fixed_site_fp64<MODE, IN>(a, i, r0 + r, o);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[r].c[c] = make_double2(o[2 * c], o[2 * c + 1]);
-    }
+    const FxForm fm = {s[r].E, fat[r], odd[r]};
+    if (form != nullptr) *form = fm;
+    else if (active[r]) fixed_site_again<MODE, IN>(fm, a, i, r0 + r, acc[r]);
   }
 }
 
@@ -985,7 +1061,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
 #pragma unroll
   for (int r = 0; r < NR; ++r) zero(acc[r]);
   constexpr int IN = GATED && MODE == MODE_PLAIN ? IN_XS : IN_HALF;  // RECON_FIXED
-  bool odd = false;
+  FxForm form = {0, 0, false};
 
   if (valid) {
     const SiteCoords sc = site_coords(g, a.out_parity, i);
@@ -995,7 +1071,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
       multi_hops<RECON, NR, MODE, kEarly>(a, ls, sc, i, r0, active, acc, dyn_smem, vbuf);
       if constexpr (EpiStage<MODE, RECON, NR>::V > 0) cp_async_wait<0>();
     } else if constexpr (RECON == RECON_FIXED) {
-      if constexpr (SPLIT) fixed_hops<NR, MODE, IN>(a, ls, sc, i, r0, active, acc, threadIdx.x / 32, 4, &odd);
+      if constexpr (SPLIT) fixed_hops<NR, MODE, IN>(a, ls, sc, i, r0, active, acc, threadIdx.x / 32, 4, &form);
       else fixed_hops<NR, MODE, IN>(a, ls, sc, i, r0, active, acc);
     } else if constexpr (PREC == PREC_F64 && NR == 1) {
       pair_hops<PREC, RECON, NR, MODE>(a, ls, sc, i, r0, active, acc);
@@ -1041,7 +1117,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
 
   if constexpr (SPLIT) {
     __shared__ double part[3][6][32];
-    __shared__ bool part_odd[3][32];
+    __shared__ FxForm part_form[3][32];
     const int dir = threadIdx.x / 32, lane = threadIdx.x & 31;
     if (dir > 0) {
 #pragma unroll
@@ -1049,7 +1125,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
         part[dir - 1][2 * c][lane] = acc[0].c[c].x;
         part[dir - 1][2 * c + 1][lane] = acc[0].c[c].y;
       }
-      part_odd[dir - 1][lane] = odd;
+      part_form[dir - 1][lane] = form;
     }
     __syncthreads();
     if (dir == 0) {
@@ -1060,17 +1136,13 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const unsigned 
           acc[0].c[c].x += part[k][2 * c][lane];
           acc[0].c[c].y += part[k][2 * c + 1][lane];
         }
-        odd |= part_odd[k][lane];
+        const FxForm p = part_form[k][lane];
+        form = {max(form.e, p.e), max(form.fat, p.fat), form.odd || p.odd};
       }
     }
     __syncthreads();  // the next item writes them again
     if (dir > 0) return;
-    if (odd) {
-      double o[6];
-      fixed_site_fp64<MODE, IN>(a, i, r0, o);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[0].c[c] = make_double2(o[2 * c], o[2 * c + 1]);
-    }
+    fixed_site_again<MODE, IN>(form, a, i, r0, acc[0]);
   }
 
   if constexpr (MODE == MODE_PLAIN) {

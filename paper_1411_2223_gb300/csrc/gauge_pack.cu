@@ -38,26 +38,29 @@ __device__ __forceinline__ void dagger(cd m[9]) {
 }
 
 __global__ void gauge_stats_kernel(const cd *fat, const cd *lng, long nlinks, double inv_s,
-                                   unsigned long long *out /* [fat max, long max, recon err, min] */) {
+                                   unsigned long long *out /* [fat max, long max, recon err, mins] */) {
   long k = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  double fm = 0, lm = 0, err = 0, least = __longlong_as_double(0x7ff0000000000000ll);
+  const double inf = __longlong_as_double(0x7ff0000000000000ll);
+  double fm = 0, lm = 0, err = 0, fleast = inf, lleast = inf;
   for (; k < nlinks; k += (long)gridDim.x * blockDim.x) {
     const cd *f = fat + k * 9;
     const cd *l = lng + k * 9;
     cd w[9];
     double pf = 0, pl = 0;
-    bool finite = true;
+    bool ffin = true, lfin = true;
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       const cd v = f[e];
       pf = fmax(pf, fmax(fabs(v.x), fabs(v.y)));
       w[e] = l[e];
       pl = fmax(pl, fmax(fabs(w[e].x), fabs(w[e].y)));
-      finite &= isfinite(v.x) && isfinite(v.y) && isfinite(w[e].x) && isfinite(w[e].y);
+      ffin &= isfinite(v.x) && isfinite(v.y);
+      lfin &= isfinite(w[e].x) && isfinite(w[e].y);
     }
     fm = fmax(fm, pf);
     lm = fmax(lm, pl);
-    least = fmin(least, finite ? fmax(pf, pl) : 0.0);
+    fleast = fmin(fleast, ffin ? pf : 0.0);
+    if (!lfin || pl > 0) lleast = fmin(lleast, lfin ? pl : 0.0);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
@@ -70,7 +73,8 @@ __global__ void gauge_stats_kernel(const cd *fat, const cd *lng, long nlinks, do
   atomic_max_pos(out + 0, fm);
   atomic_max_pos(out + 1, lm);
   atomic_max_pos(out + 2, err);
-  atomicMax(out + 3, ~(unsigned long long)__double_as_longlong(least));
+  atomicMax(out + 3, ~(unsigned long long)__double_as_longlong(fleast));
+  atomicMax(out + 4, ~(unsigned long long)__double_as_longlong(lleast));
 }
 
 __device__ __forceinline__ uint32_t link_word(cd v, float inv) {
@@ -92,11 +96,15 @@ __device__ void store_pairs(char *links, int S, int i, int mu, const cd ff[9], c
       const int2 re = fx_link_word(v.x, ps.to_fixed), im = fx_link_word(v.y, ps.to_fixed);
       return make_int4(re.x, re.y, im.x, im.y);
     };
+    auto long_word = [&](cd v) {
+      const int2 re = fx_long_word(v.x, ps.to_fixed), im = fx_long_word(v.y, ps.to_fixed);
+      return make_int4(re.x, re.y, im.x, im.y);
+    };
     for (int k = 0; k < 9; ++k) {
       pf[(size_t)k * S + i] = word(ff[k]);
       pf[(size_t)(9 + k) * S + i] = word(fb[k]);
-      pl[(size_t)k * S + i] = word(lf[k]);
-      pl[(size_t)(9 + k) * S + i] = word(lb[k]);
+      pl[(size_t)k * S + i] = long_word(lf[k]);
+      pl[(size_t)(9 + k) * S + i] = long_word(lb[k]);
     }
   } else if constexpr (PREC == PREC_F64) {
     double2 *pf = reinterpret_cast<double2 *>(fat);

@@ -15,10 +15,11 @@ struct PackScales {
 
 // Per-field maxima over nlinks = 4V links: out[0] = max |re|,|im| of fat,
 // out[1] = same for long, out[2] = max deviation of the long links' third row
-// from inv_s * conj(row0 x row1), out[3] = the complement of the bits of the
-// smallest, over the (site, direction) pairs, of the larger of the pair's two
-// links' maxima (of 0 for a pair with an element that is not finite).  out
-// holds non-negative doubles as u64 bits and must be zeroed by the caller.
+// from inv_s * conj(row0 x row1), out[3] and out[4] = the complement of the bits
+// of the smallest of the fat links' own maxima and of the long links' (of those
+// that are not zero; infinity if all are; 0 where a link has an element that is
+// not finite).  out holds non-negative doubles as u64 bits and must be zeroed by
+// the caller.
 int launch_gauge_stats(const double *fat, const double *lng, long nlinks, double inv_s,
                        unsigned long long *out, cudaStream_t st);
 

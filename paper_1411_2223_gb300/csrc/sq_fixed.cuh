@@ -9,15 +9,31 @@
 // colour vectors: one per output site, raised while its 16 neighbours are
 // read), and a product is three integer multiply-adds into two 64-bit sums,
 //   hi += ah bh,   mid += ah bl + al bh,
-// exact but for the term al bl (below 2^-54 of the blocks' scales).  The sums
-// over the 96 real products of an output component neither round nor
-// overflow:
+// exact but for the term al bl (2^-57 of the blocks' scales at most), which is
+// dropped.  The sums over the 96 real products of an output component neither
+// round nor overflow:
 //   |hi| <= 96 2^56 < 2^63,  |mid| <= 96 (2^28 2^27 + 2^26 2^28) < 2^63
 // (the links' low words are balanced, |al| <= 2^26).  The result is rounded to
 // FP64 once; a chain of FP64 FMAs rounds at each of its 96 steps.  Against a
 // long-double Dslash of Gaussian vectors the 2-norm error is 1.5e-16, with
 // FP64 FMAs 3.5e-16 (2.7e-16 against 3.5e-16 where neighbouring sites differ
 // by factors up to e^8), the largest error of a component 5e-16 against 2e-15.
+//
+// The long links are 24 times smaller than the fat ones as a rule, and have 50 of
+// the 55 bits; a neighbour much smaller than the site's largest has fewer too.
+// That is enough beside the terms of the fat links and the larger neighbours, but
+// not where the vector reaches a site by the long links only, or almost (point and
+// wall sources, steep decays): such sites, told by the exponents of the vectors,
+// are computed again with the two kinds apart, for which the long links' words
+// hold FX_MORE more bits.  Rms over the sites of the error relative to the site, a
+// point source's long-hop sites 2.0e-15 -> 8.8e-17; Gaussian vectors that decay in
+// t as exp(-k |t|), 8^3 x 16, against a C Dslash in FP64:
+//   k            0        0.5      0.7      1        1.5      2        3
+//   before       1.9e-16  2.4e-16  3.2e-16  5.9e-16  1.5e-15  2.2e-15  2.3e-15
+//   here         1.9e-16  2.3e-16  2.6e-16  2.5e-16  2.2e-16  2.3e-16  2.2e-16
+//   FP64 FMAs    1.9e-16  1.9e-16  1.8e-16  1.7e-16  1.5e-16  1.3e-16  1.2e-16
+// dirac_apply at 20^3 x 64: 221 us, with a point source 202, a wall 268, and 585
+// where every site is computed again (k = 1; with FP64 FMAs 867 for any vector).
 //
 // What it bounds: the FP64 Dslash of one system at 20^3 x 64 went from
 // 321.6 us (FP64 units 100 % busy) to 110 us, 0.84 of the HBM rate for its
@@ -33,6 +49,16 @@ namespace sq {
 constexpr int FX_LOW = 27;                 // bits of a low word
 constexpr int FX_BITS = 55;                // bits of a value
 constexpr int FX_LOW_MASK = (1 << FX_LOW) - 1;
+constexpr int FX_MORE = 5;                 // further bits of a long link
+// A nonzero link's largest element is at least 2^-FX_FAT_LEAST (fat) or
+// 2^-FX_LONG_LEAST (long) of the field's scale, and so held to 2^-51 of itself.
+constexpr int FX_FAT_LEAST = 5, FX_LONG_LEAST = 9;
+// How far the exponent of a site's largest fat-hop neighbour may be below that of
+// all its neighbours: at most 8 times smaller, which costs 2.6e-16 (table above).
+// In Gaussian vectors they are never further apart (all 48 components by fat hops
+// 4 times smaller than one by long hops: some 10^-9 of the sites); with 1 here the
+// sites of random fields that are cost 19 % of the time.
+constexpr int FX_KINDS_APART = 2;
 // Biased FP64 exponents the fixed-point path takes: below FX_MIN_E a vector
 // counts as zero at every scale in use, from FX_MAX_E on (which includes
 // infinities and NaN) the site is computed with FP64 FMAs.
@@ -141,6 +167,29 @@ __device__ __forceinline__ void fx_mat_vec(FxAcc &a, const int4 (&m)[9], const F
   }
 }
 
+// Colour c of the vector v (XS: v + d) relative to E, times sgn.
+template <bool XS>
+__device__ __forceinline__ void fx_colour(const Vec3<double> &v, const Vec3<double> &d, int E, int sgn,
+                                          int c, Fx &re, Fx &im) {
+  re = fx_from_double(v.c[c].x, E, sgn);
+  im = fx_from_double(v.c[c].y, E, sgn);
+  if (XS) {
+    const Fx p = fx_from_double(d.c[c].x, E, sgn), q = fx_from_double(d.c[c].y, E, sgn);
+    const int lr = re.l + p.l, li = im.l + q.l;
+    re.h += p.h + (lr >> FX_LOW);
+    re.l = lr & FX_LOW_MASK;
+    im.h += q.h + (li >> FX_LOW);
+    im.l = li & FX_LOW_MASK;
+  }
+}
+
+// Products are in units of 2^(fixed_exp - FX_BITS) 2^(E - 1022 - FX_BITS), the
+// sums' hi of 2^(2 FX_LOW) of these: that unit.
+__device__ __forceinline__ double fx_unit(int fixed_exp, int E) {
+  const int ex = fixed_exp + E - 1022 - 2 * FX_BITS + 2 * FX_LOW;
+  return __hiloint2double((ex + 1023) << 20, 0);
+}
+
 // (hi 2^27 + mid) 2^27 in units of the operands' last bits, times `unit`
 __device__ __forceinline__ double fx_to_double(long long hi, long long mid, double unit) {
   const double d = (double)(hi + (mid >> FX_LOW));
@@ -153,6 +202,20 @@ __device__ __forceinline__ int2 fx_link_word(double v, double to_fixed) {
   const long long q = __double2ll_rn(v * to_fixed);
   const long long h = (q + (1ll << (FX_LOW - 1))) >> FX_LOW;
   return make_int2((int)(q - (h << FX_LOW)), (int)h);
+}
+// Of a long link: the low word 2^FX_MORE l + x, x = 0 .. 2^FX_MORE - 1 the further
+// bits with half of their range added, so that a shift gives the rounded l.
+__device__ __forceinline__ int2 fx_long_word(double v, double to_fixed) {
+  constexpr int half = 1 << (FX_MORE - 1);
+  const long long more = __double2ll_rn(v * (to_fixed * (1 << FX_MORE))) + half;
+  const long long q = more >> FX_MORE, h = (q + (1ll << (FX_LOW - 1))) >> FX_LOW;
+  return make_int2((int)(more - (h << (FX_LOW + FX_MORE))), (int)h);
+}
+__device__ __forceinline__ int4 fx_long_element(int4 q) {
+  return make_int4(q.x >> FX_MORE, q.y, q.z >> FX_MORE, q.w);
+}
+__device__ __forceinline__ int fx_long_rest(int l) {
+  return (l & ((1 << FX_MORE) - 1)) - (1 << (FX_MORE - 1));
 }
 
 }  // namespace sq

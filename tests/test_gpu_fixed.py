@@ -236,3 +236,95 @@ def test_dirac_apply_on_overlapping_vectors(sq, shift):
         assert rel(dst.cpu().numpy(), want.cpu().numpy()) <= 1e-15
     finally:
         sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('long_scale', [1.0, 2.0 ** -2, 2.0 ** -14, 2.0 ** -30, 2.0 ** 5, 'half', 0.0])
+def test_point_source_site_by_site(sq, long_scale):
+    """Every site that a point source reaches, relative to itself: on 8^4 each
+    is reached by one hop.  A fat link's elements are off by 2^-55 (the fields'
+    largest is 1.1 to 1.4), that is 3 sqrt(2) 2^-55 of the result at most, and the
+    result by 2^-53; long links of 1/96 to 4/3 are held to 2^-60, or 2^-53 of
+    3 sqrt(2) times themselves, and FP64 FMAs add 3 2^-53: below 2^-51.  Long links
+    of zero ('half': of half the sites) are exact."""
+    dims = (8, 8, 8, 8)
+    fat, lng = (a.copy() for a in gauge(dims))
+    if long_scale == 'half':
+        lng[::2] = 0.0
+    else:
+        lng *= long_scale
+    vol = oracle.volume(dims)
+    vh = vol // 2
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        for p in (0, 1):
+            v = np.zeros((vh, 3), dtype=np.complex128)
+            v[901] = synth.gaussian_source(vh, 3)[901]
+            want = _reference(dims, fat, lng, v, p).astype(np.complex128)
+            size = np.linalg.norm(want, axis=1)
+            got = gpu_dslash(sq, gid, 'f64', 18, v, p, vh)
+            assert np.all(np.linalg.norm(got - want, axis=1) <= 2.0 ** -51 * size)
+            full = np.zeros((vol, 3), dtype=np.complex128)
+            full[oracle.half_sites(dims, 1 - p)] = v
+            out = to_dev(np.full_like(full, np.nan))
+            sq.dirac_apply(gid, 0.0, to_dev(full), out)
+            got = out.cpu().numpy()[oracle.half_sites(dims, p)]
+            assert np.all(np.linalg.norm(got - want, axis=1) <= 2.0 ** -51 * size)
+    finally:
+        sq.gauge_free(gid)
+
+
+@pytest.mark.parametrize('decay', [0.0, 0.7, 1.5, 3.0])
+def test_steep_decays_site_by_site(sq, decay):
+    """Neighbours by long hops exp(2 decay) times larger than those by fat hops:
+    a fat-hop neighbour at most 8 times smaller is cut at 2^-53 of the larger
+    one's size, uniformly, and six parts enter a component, which is
+    sqrt(6 / 3) 8 2^-54 = 2^-50.5 of it (rms); past 8 both kinds keep an exponent
+    of their own.  The rms over the sites of the error relative to the site stays
+    below 2^-50."""
+    dims = (8, 8, 8, 16)
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        for p in (0, 1):
+            t = oracle.half_sites(dims, 1 - p) // 512
+            v = synth.gaussian_source(vh, 5) * np.exp(-decay * np.minimum(t, 16 - t))[:, None]
+            want = _reference(dims, fat, lng, v, p)
+            got = gpu_dslash(sq, gid, 'f64', 18, v, p, vh)
+            err = np.linalg.norm((got - want).astype(np.complex128), axis=1)
+            err /= np.linalg.norm(want.astype(np.complex128), axis=1)
+            assert np.sqrt(np.mean(err ** 2)) <= 2.0 ** -50
+    finally:
+        sq.gauge_free(gid)
+
+
+# sites per parity that the resident kernel takes with four, two and one lane
+@pytest.mark.parametrize('dims', [(4, 4, 4, 8), (12, 14, 14, 24), (16, 16, 16, 32)])
+def test_point_source_solves(sq, dims):
+    """A point source sends its surroundings through the site-by-site form in the
+    operator's tiles, the resident kernel and the reliable updates: tiles give
+    the bits of one system, and solves the residual they report (as
+    test_reliable_updates_of_one_system)."""
+    import torch
+    fat, lng = gauge(dims)
+    vh = oracle.volume(dims) // 2
+    b = np.zeros((vh, 3), dtype=np.complex128)
+    b[vh // 3] = synth.gaussian_source(vh, 3)[vh // 3]
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        nbytes, _ = sq.spinor_bytes(gid, 'f64')
+        src = torch.zeros((5, nbytes), dtype=torch.uint8, device='cuda')
+        out, one = torch.zeros_like(src), torch.zeros_like(src)
+        for j in range(5):
+            sq.pack_spinor(gid, 'f64', to_dev(np.roll(b, 7 * j, axis=0)), src[j])
+            sq.dslash_apply(gid, 1, 'f64', 18, src[j], one[j])
+        sq.dslash_apply_multi(gid, 1, 'f64', 18, 5, src, out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, one)
+        for prec in ('f64', 'f32', 'i16'):
+            x, st = sq.cg_solve(gid, b, 0.5, 1e-9, precision=prec)
+            assert st['status'] == 0
+            true = oracle.true_residual(dims, fat, lng, 0.5, b, x)
+            assert true <= 1e-9 and abs(st['true_residual'] - true) <= 1e-12
+    finally:
+        sq.gauge_free(gid)
