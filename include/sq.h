@@ -114,11 +114,11 @@ typedef struct {
     double seconds;        /* wall time of the solve (host clock)              */
     double gflops;         /* 2364 flop per even site per iteration            */
     /* Launch shapes of the CG's two sloppy Dslash kernels as launched (the
-     * tuner's choice, or a SQ_TUNE_CACHE entry): threads per block and
+     * tuner's choice, or one that SQ_TUNE_CACHE forces): threads per block and
      * right-hand sides per thread of the D_oe kernel (with the reduction)
      * and of the D_eo kernel (with the update).  A single system on a lattice of
      * up to 512 sites per parity and SM runs as one resident kernel instead,
-     * unless a SQ_TUNE_CACHE entry gives these shapes: then its threads per
+     * unless SQ_TUNE_CACHE forces one of these shapes: then its threads per
      * block and 1.  0 where no batched CG ran. */
     int oe_block, oe_rhs_tile, eo_block, eo_rhs_tile;
 } sq_cg_stats;
@@ -304,12 +304,16 @@ int dslash_apply_multi(sq_ctx *ctx, int gauge_id, int out_parity, int prec, int 
  * gauge field: threads per block and right-hand sides per thread, for `nrhs`
  * systems in `prec` with `long_recon`-real long links.  mode: 0 the plain
  * Dslash (dslash_apply, dslash_apply_multi, the FP64 reliable-update pair),
- * 1 with the m^2 epilogue (mdagm_apply, multi-shift), 3 the CG's D_oe kernel
- * with its reduction, 4 the CG's D_eo kernel with its update.  The shape is
- * chosen by timing the candidates on first use (which allocates scratch and
- * synchronises `stream`) unless SQ_TUNE_CACHE or an earlier call fixed it;
- * for modes 1, 3 and 4, which run in chains of dependent launches, the
- * smallest block within 3 % of the fastest is taken.
+ * 1 with the m^2 epilogue, 3 the CG's and the multi-shift phase's D_oe kernel
+ * with its reduction, 4 their D_eo kernel with its update.  The shape is chosen
+ * by timing the candidates on first use (which allocates scratch and
+ * synchronises `stream`) unless an earlier call did so, or one of an earlier
+ * process in the file that the environment variable SQ_TUNE_CACHE names; for
+ * modes 1, 3 and 4, which run in chains of dependent launches, the smallest
+ * block within 3 % of the fastest is taken.  A line
+ *   dslash_v4:<Lx>x<Ly>x<Lz>x<Lt>:p<prec>:r<long_recon>:n<nrhs>:m<mode> <block> <rhs_tile>
+ * of the file forces a shape (files of older versions consist of such lines);
+ * the tuner's own lines begin with dslash_v5 and force nothing.
  * (The paper's QUDA path tunes its launches at run time, Sec. 3.) */
 int sq_tuned_launch(sq_ctx *ctx, int gauge_id, int prec, int long_recon, int nrhs, int mode,
                     void *stream, int *block, int *rhs_tile);

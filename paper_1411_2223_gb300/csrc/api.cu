@@ -594,9 +594,9 @@ int solve_batch_locked(sq_ctx *ctx, int gauge_id, int nrhs, const double *src,
   if (!w) {
     int rc = cg_work_create(ctx, gf, o.precision, o.long_recon, nrhs, &w);
     if (rc) return rc;
-    // launch shapes that a tuning file gives are launched
-    if (!tuned_pinned(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_NORM) &&
-        !tuned_pinned(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_UPDATE))
+    // launch shapes that a tuning file forces are launched
+    if (!tuned_forced(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_NORM) &&
+        !tuned_forced(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_UPDATE))
       w->resident_block = cg_resident_block(w);
     if (!w->resident_block) {
       w->cfg_norm = tuned_dslash(ctx, *gf, o.precision, o.long_recon, nrhs, MODE_NORM, st);

@@ -98,8 +98,8 @@ struct DslashConfig {
 
 DslashConfig tuned_dslash(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs,
                           int mode, cudaStream_t st);
-// Is the shape given by the file SQ_TUNE_CACHE named?
-bool tuned_pinned(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs, int mode);
+// Does a user's line of the file SQ_TUNE_CACHE force the shape?
+bool tuned_forced(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs, int mode);
 Tuner *tuner_create();
 void tuner_destroy(Tuner *);
 

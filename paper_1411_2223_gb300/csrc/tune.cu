@@ -4,14 +4,13 @@
 // (Sec. 3); this tuner times every candidate with CUDA events on the first
 // use of a (lattice, precision, link format, batch size) key and caches the
 // winner for the context.  SQ_TUNE_CACHE=<file> persists the cache across
-// processes.
+// processes; lines that a user puts there force their shapes.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <fstream>
 #include <map>
 #include <mutex>
-#include <set>
 #include <sstream>
 #include <string>
 #include <utility>
@@ -24,15 +23,27 @@ namespace sq {
 struct Tuner {
   std::mutex mu;
   std::map<std::string, DslashConfig> cache;
-  std::set<std::string> pinned;  // keys read from the file
+  std::map<std::string, DslashConfig> forced;  // the user's lines of the file
   std::string path;
 };
 
-static std::string tune_key(const Geom &g, int prec, int recon, int nrhs, int mode) {
+// A user's line of the file and a choice of the tuner have different names, so
+// that what the library has written there itself forces nothing on a later
+// process.  The FP64 kernels of fields with fixed-point links (:x) and with
+// doubles (:d) are different ones.
+constexpr char FORCED[] = "dslash_v4:", CHOSEN[] = "dslash_v5:";
+static std::string shape_key(const Geom &g, int prec, int recon, int nrhs, int mode) {
   std::ostringstream s;
-  s << "dslash_v4:" << g.L[0] << "x" << g.L[1] << "x" << g.L[2] << "x" << g.L[3] << ":p" << prec
-    << ":r" << recon << ":n" << nrhs << ":m" << mode;
+  s << g.L[0] << "x" << g.L[1] << "x" << g.L[2] << "x" << g.L[3] << ":p" << prec << ":r" << recon
+    << ":n" << nrhs << ":m" << mode;
   return s.str();
+}
+static std::string forced_key(const GaugeField &gf, int prec, int recon, int nrhs, int mode) {
+  return FORCED + shape_key(gf.g, prec, recon, nrhs, mode);
+}
+static std::string chosen_key(const GaugeField &gf, int prec, int recon, int nrhs, int mode) {
+  const char *form = prec != PREC_F64 ? "" : gf.scales(prec, recon).fixed ? ":x" : ":d";
+  return CHOSEN + shape_key(gf.g, prec, recon, nrhs, mode) + form;
 }
 
 Tuner *tuner_create() {
@@ -43,27 +54,24 @@ Tuner *tuner_create() {
     std::ifstream in(t->path);
     std::string key;
     DslashConfig c;
-    while (in >> key >> c.block >> c.nr) {
-      t->cache[key] = c;
-      t->pinned.insert(key);
-    }
+    while (in >> key >> c.block >> c.nr)
+      (key.rfind(FORCED, 0) == 0 ? t->forced : t->cache)[key] = c;
   }
   return t;
 }
 
 void tuner_destroy(Tuner *t) { delete t; }
 
-bool tuned_pinned(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs, int mode) {
-  Tuner *t = ctx->tuner;
-  if (!t) return false;
-  std::lock_guard<std::mutex> lk(t->mu);
-  return t->pinned.count(tune_key(gf.g, prec, recon, nrhs, mode)) != 0;
+bool tuned_forced(sq_ctx *ctx, const GaugeField &gf, int prec, int recon, int nrhs, int mode) {
+  Tuner *t = ctx->tuner;  // `forced` does not change after the start
+  return t && t->forced.count(forced_key(gf, prec, recon, nrhs, mode)) != 0;
 }
 
 static void tuner_save(Tuner *t) {
   if (t->path.empty()) return;
   std::ofstream out(t->path);
-  for (auto &kv : t->cache) out << kv.first << " " << kv.second.block << " " << kv.second.nr << "\n";
+  for (auto *m : {&t->forced, &t->cache})
+    for (auto &kv : *m) out << kv.first << " " << kv.second.block << " " << kv.second.nr << "\n";
 }
 
 // Device buffers and arguments of one Dslash kernel on synthetic inputs, for
@@ -181,7 +189,9 @@ DslashConfig tuned_dslash(sq_ctx *ctx, const GaugeField &gf, int prec, int recon
   def.nr = nrhs >= 4 ? 4 : nrhs >= 2 ? 2 : 1;
   Tuner *t = ctx->tuner;
   if (!t || !gf.has(prec, recon)) return def;
-  const std::string key = tune_key(gf.g, prec, recon, nrhs, mode);
+  const auto forced = t->forced.find(forced_key(gf, prec, recon, nrhs, mode));
+  if (forced != t->forced.end()) return forced->second;
+  const std::string key = chosen_key(gf, prec, recon, nrhs, mode);
   std::lock_guard<std::mutex> lk(t->mu);
   auto it = t->cache.find(key);
   if (it != t->cache.end()) return it->second;
