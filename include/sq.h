@@ -186,10 +186,11 @@ int gauge_fatten(sq_ctx *ctx, const int dims[4], const double *thin_dev, double 
  * tree-level asqtad values are {5/8, 1/16, 1/64, 1/384, -1/16, -1/24}, which
  * give 9/8 and -1/24 on unit links.  The paper's lattices are MILC asqtad
  * ensembles (Sec. 2, Fig. 1).  Arrays and `stream` as for gauge_fatten; the
- * paths are built as nested staple fields in a stream-ordered device scratch
- * of 2736 bytes per site, taken and returned on `stream` (outside the HBM
- * budget); where the device refuses that much, the lattice is done in slabs of
- * time slices with a part of it. */
+ * paths are built as nested staple fields in a stream-ordered device scratch,
+ * taken and returned on `stream` and not counted in the HBM budget: 2736 bytes
+ * per site; where that is more than is left of the budget, or the device refuses
+ * it, the lattice is done in slabs of slices across its longest direction (L
+ * slices), down to 7 / L of it.  Results do not depend on that. */
 int gauge_fatten_asqtad(sq_ctx *ctx, const int dims[4], const double *thin_dev,
                         const double coeffs[6], double *fat_dev, double *lng_dev, void *stream);
 

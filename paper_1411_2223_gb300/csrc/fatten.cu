@@ -180,12 +180,16 @@ struct FatScale {
   unsigned uneven;             // a link is not unitary
 };
 
-// Time slices in scratch: slot (t - t0) mod Lt, slots 0 .. nslots - 1.
+// Slices of the lattice across direction `ax` in scratch: slot (t - t0) mod L for
+// the slice at coordinate t, slots 0 .. nslots - 1; in a slice the other three
+// directions in their order.
 struct Slab {
   FatGeom g;
+  int ax, od[3];               // the slices' direction, and the others
+  long st[4];                  // scratch strides of the others
   int t0, nslots;
   int first, count;            // slots a kernel writes
-  long v3;                     // sites of a time slice
+  long v3;                     // sites of a slice
   long n;                      // scratch sites: nslots * v3
 };
 
@@ -224,14 +228,16 @@ __device__ __forceinline__ bool slab_site(const Slab &sl, SlabSite &p) {
   const int r3 = (int)(idx - dt * sl.v3);
   const int slot = sl.first + dt;
   int t = sl.t0 + slot;
-  if (t >= sl.g.L[3]) t -= sl.g.L[3];
-  int r = r3;
-  p.c[0] = r % sl.g.L[0]; r /= sl.g.L[0];
-  p.c[1] = r % sl.g.L[1];
-  p.c[2] = r / sl.g.L[1];
-  p.c[3] = t;
+  if (t >= sl.g.L[sl.ax]) t -= sl.g.L[sl.ax];
+  const int l0 = sl.g.L[sl.od[0]], l1 = sl.g.L[sl.od[1]];
+  const int c0 = r3 % l0, q = r3 / l0, c1 = q % l1, c2 = q / l1;
+  p.lex = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    p.c[k] = k == sl.ax ? t : k == sl.od[0] ? c0 : k == sl.od[1] ? c1 : c2;
+    p.lex += p.c[k] * sl.g.st[k];
+  }
   p.s = slot * sl.v3 + r3;
-  p.lex = t * sl.v3 + r3;
   return true;
 }
 
@@ -246,8 +252,8 @@ __device__ __forceinline__ SlabSite slab_step(const Slab &sl, const SlabSite &y,
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if (k == mu) z.c[k] = v;
-  if (mu < 3) {
-    z.s = y.s + (long)(v - cy) * sl.g.st[mu];
+  if (mu != sl.ax) {
+    z.s = y.s + (long)(v - cy) * sl.st[mu];
   } else {  // whole lattice in scratch: the wrap; else the next slot
     long s = y.s + d * sl.v3;
     if (s < 0) s += sl.n;
@@ -641,7 +647,17 @@ extern "C" int gauge_fatten_asqtad(sq_ctx *ctx, const int dims[4], const double 
   const double2 *u = reinterpret_cast<const double2 *>(thin_dev);
   AsqtadArgs a{};
   a.sl.g = make_fat_geom(dims, vol);
-  a.sl.v3 = vol / dims[3];
+  auto slices = [&](int ax) {
+    a.sl.ax = ax;
+    a.sl.v3 = vol / dims[ax];
+    long s = 1;
+    for (int k = 0, j = 0; k < 4; ++k)
+      if (k != ax) {
+        a.sl.od[j++] = k;
+        a.sl.st[k] = s;
+        s *= dims[k];
+      }
+  };
   a.fat = reinterpret_cast<double2 *>(fat_dev);
   a.c1 = k.one;
   a.c3 = k.three;
@@ -658,27 +674,38 @@ extern "C" int gauge_fatten_asqtad(sq_ctx *ctx, const int dims[4], const double 
   a.f7 = fat_coef(k.seven, 1 - FX_BITS, E);
   a.fl = fat_coef(k.lepage, -FX_BITS, E);
   a.w_unit = std::ldexp(1.0, E - FX_BITS - 2);
-  // Scratch of a time slice's site: 36 link planes, 6 S, 3 A and 6 W fields of 9
-  // planes, 16 bytes each.  The whole lattice at once where that can be had;
-  // else slabs of nt slices, with the slices their staples reach: links to 3,
-  // S and A to 2, W to 1 slices beyond (the Naik link reaches 2).
-  const size_t slice_b = (size_t)a.sl.v3 * 16 * (36 + 54 + 27 + 54);
-  const size_t head = 256;
+  // Scratch of a site: 36 link planes, 6 S, 3 A and 6 W fields of 9 planes, 16
+  // bytes each.  The whole lattice at once where that is within what is left of
+  // the context's budget and can be had; else slabs of nt slices across the
+  // longest direction, with the slices their staples reach: links to 3, S and A
+  // to 2, W to 1 slices beyond (the Naik link reaches 2).  The smallest slab, of
+  // one slice and 7 slots, is taken whatever is left, and lattices with no
+  // direction longer than 7 (1296 sites at most) are done whole.
+  const size_t site_b = 16 * (36 + 54 + 27 + 54), head = 256;
+  size_t left;
+  {
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    left = ctx->budget > ctx->in_use ? ctx->budget - ctx->in_use : 0;
+  }
+  int longest = 3;
+  for (int k = 2; k >= 0; --k)
+    if (dims[k] > dims[longest]) longest = k;
+  bool whole = dims[longest] <= 7 || head + site_b * vol <= left;
   void *scratch = nullptr;
-  int nt = dims[3];
-  bool whole = true;
+  int nt = 0;
   for (;;) {
-    const int slots = whole ? dims[3] : nt + 6;
-    const cudaError_t me = cudaMallocAsync(&scratch, head + slice_b * slots, st);
-    if (me == cudaSuccess) {
-      a.sl.nslots = slots;
-      break;
-    }
+    slices(whole ? 3 : longest);
+    const size_t slice_b = site_b * a.sl.v3;
+    if (whole) nt = dims[3];
+    else if (nt == 0) nt = (int)std::min<size_t>(std::max<size_t>(left / slice_b, 7) - 6, dims[longest] - 7);
+    a.sl.nslots = whole ? nt : nt + 6;
+    const cudaError_t me = cudaMallocAsync(&scratch, head + slice_b * a.sl.nslots, st);
+    if (me == cudaSuccess) break;
     if (me != cudaErrorMemoryAllocation) SQ_CUDA_TRY(me);
     cudaGetLastError();
-    nt = whole ? (dims[3] - 7) : nt / 2;
+    nt = whole ? 0 : nt / 2;
+    if ((whole && dims[longest] <= 7) || (!whole && nt < 1)) SQ_CUDA_TRY(me);
     whole = false;
-    if (nt < 1) SQ_CUDA_TRY(me);
   }
   a.sl.n = a.sl.nslots * a.sl.v3;
   FatScale *sc = static_cast<FatScale *>(scratch);
@@ -693,7 +720,7 @@ extern "C" int gauge_fatten_asqtad(sq_ctx *ctx, const int dims[4], const double 
     fat_scale_kernel<<<8 * ctx->sms, 256, 0, st>>>(u, 4 * vol, sc);
     ctx->launches++;
   }
-  const int Lt = dims[3];
+  const int Lt = dims[a.sl.ax];
   for (int t = 0; t < Lt && e == cudaSuccess; t += nt) {
     const int m = std::min(nt, Lt - t);       // slices finished by this slab
     const int halo = whole ? 0 : 3;

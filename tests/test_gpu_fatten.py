@@ -249,3 +249,36 @@ def test_asqtad_links_with_unit_rows_that_are_not_unitary(sq, what):
     for got, want in ((fat.cpu().numpy(), f0), (lng.cpu().numpy(), l0)):
         assert rel(got, want) <= 2e-15
         assert np.abs(got - want).max() <= 1e-14 * np.abs(want).max()
+
+
+@pytest.mark.parametrize('unitary', [True, False])
+@pytest.mark.parametrize('dims', [(4, 2, 4, 16), (4, 2, 14, 4), (2, 12, 4, 12), (10, 4, 2, 4), (2, 2, 2, 8),
+                                  (6, 4, 2, 6)])
+def test_asqtad_slabs_give_the_bits_of_the_whole_lattice(sq, dims, unitary):
+    """Where the scratch is more than is left of the budget the lattice is done in
+    slabs across its longest direction: of one slice, of two, of as many as leave
+    a part of one at the end, of all but the halo's worth; the first and the last
+    wrap around.  The same sums, so the same bits."""
+    import torch
+    from paper_1411_2223_gb300 import sq as sqm
+    u = synth.thin_links(dims, 0.7, 6)
+    if not unitary:
+        u = u * np.random.default_rng(3).uniform(0.5, 2, u.shape[:2])[..., None, None]
+    t = torch.from_numpy(u).cuda()
+    want = [torch.empty_like(t) for _ in range(2)]
+    sq.gauge_fatten_asqtad(dims, t, *want)
+    assert rel(want[0].cpu().numpy(), _asqtad_ref(dims, u, sq.ASQTAD_COEFFS)[0]) <= 2e-15
+    longest = max(dims)
+    slice_bytes = 2736 * (oracle.volume(dims) // longest)
+    for nt in sorted({1, 2, 3, longest - 7}):
+        if nt < 1 or nt > max(longest - 7, 1):
+            continue
+        with sqm.Context(0, hbm_budget=slice_bytes * (nt + 6) + slice_bytes // 2) as ctx:
+            got = [torch.full_like(t, float('nan')) for _ in range(2)]
+            torch.cuda.synchronize()
+            n = ctx.kernel_launches()
+            ctx.gauge_fatten_asqtad(dims, t, *got)
+            torch.cuda.synchronize()
+            slabs = 1 if longest <= 7 else -(-longest // nt)
+            assert ctx.kernel_launches() - n == 1 + 27 * slabs
+        assert all(torch.equal(g, w) for g, w in zip(got, want))
