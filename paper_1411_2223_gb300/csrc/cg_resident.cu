@@ -324,6 +324,15 @@ __global__ void __launch_bounds__(THREADS, 1) cg_resident_kernel(const __grid_co
   if (blockIdx.x == 0 && tid == 0) *a.norm.slots = s;
 }
 
+// Iterations of one launch: about 4 ms of them at most, as the kernel holds every
+// SM and other streams' kernels (a served batch's) get in between launches only.
+// 128 whatever the size, as it was first, were 10 ms in FP64 at 65536 sites; a new
+// launch and the empty update pair before it cost some 20 us.
+inline int resident_steps(int prec, int vh) {
+  const double us = 10.0 + vh * (prec == PREC_F64 ? 1.1e-3 : 0.45e-3);  // see the table below
+  return std::min(128, (int)(4000.0 / us));
+}
+
 // Lanes per site, and threads per block with the sites spread over the SMs in
 // whole warps: four lanes while a block stays within 512 threads.
 inline int lanes_per_site(int vh, int sms) {
@@ -403,7 +412,7 @@ int cg_enqueue_resident(CGWork *w, const DslashArgs &norm, const DslashArgs &upd
   a.count = reinterpret_cast<unsigned *>(base + 128);
   a.sums = reinterpret_cast<double *>(base + 256);
   a.p2 = base + barrier_bytes(w->ctx);
-  a.max_steps = RESIDENT_STEPS;
+  a.max_steps = resident_steps(w->prec, norm.g.vh);
   SQ_CUDA_TRY(cudaMemsetAsync(a.count, 0, sizeof(unsigned), st));
   int rc = -1;
   const int block = w->resident_block, lanes = lanes_per_site(norm.g.vh, w->ctx->sms);

@@ -146,10 +146,8 @@ int cg_enqueue_block(CGWork *w, int k, bool graph, cudaStream_t st);
 // Run until no slot is running; host polls the slot state after each block.
 int cg_run(CGWork *w, int block_iters, bool graph, cudaStream_t st);
 int cg_run_resident(CGWork *w, cudaStream_t st);
-// The one-system CG as a resident kernel (cg_resident.cu): iterations of one
-// launch (a few ms at most, so that other streams' kernels get in between),
-// and its block for a workspace it is the faster form for (else 0).
-constexpr int RESIDENT_STEPS = 128;
+// The one-system CG as a resident kernel (cg_resident.cu): the memory it needs,
+// its block for a workspace it is the faster form for (else 0), and a launch.
 size_t cg_resident_bytes(const sq_ctx *ctx, int vh, int nrhs, int prec, size_t fb);
 int cg_resident_block(const CGWork *w);
 int cg_enqueue_resident(CGWork *w, const DslashArgs &norm, const DslashArgs &update,

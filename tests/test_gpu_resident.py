@@ -102,3 +102,23 @@ def test_guess_limits_and_long_solves(sq, prec):
         assert np.array_equal(x, z)
     finally:
         sq.gauge_free(gid)
+
+
+def test_a_launch_ends_within_milliseconds(sq):
+    """FP64 at 65536 sites per parity, some 80 us an iteration: other streams get
+    the device after 4 ms, that is 64 iterations or fewer, and the solve is a
+    chain of such launches, each with the pair of an update after it (three more
+    kernels pack, start and unpack)."""
+    dims = (16, 16, 16, 32)
+    fat, lng = gauge(dims, 0.25, 0)
+    b = synth.gaussian_source(oracle.volume(dims) // 2, 4)
+    gid = sq.gauge_load(dims, fat, lng)
+    try:
+        sq.cg_solve(gid, b, 0.5, 1e-2, precision='f64')  # tunes
+        n = sq.kernel_launches()
+        x, st = sq.cg_solve(gid, b, 0.01, 1e-9, precision='f64')
+        n = sq.kernel_launches() - n
+        assert oracle.true_residual(dims, fat, lng, 0.01, b, x) <= 1e-9
+        assert st['iterations'] > 256 and (n - 3) // 3 * 64 >= st['iterations'], (n, st['iterations'])
+    finally:
+        sq.gauge_free(gid)
