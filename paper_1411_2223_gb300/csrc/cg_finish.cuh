@@ -1,5 +1,7 @@
 // Scalar steps of the CG recurrences, run by one thread of the last block of
-// each reduction kernel so that an iteration needs no host round trip.
+// each reduction kernel (the shifts' steps of a multi-shift CG by a lane of its
+// warp each; the resident kernel's by a thread of every block) so that an
+// iteration needs no host round trip.
 //
 // CG on A x = b (Hestenes-Stiefel): alpha = rr / <p, A p>, x += alpha p,
 // r -= alpha A p, beta = rr_new / rr, p = r + beta p.  The mixed-precision

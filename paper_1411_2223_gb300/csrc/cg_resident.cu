@@ -382,7 +382,8 @@ static size_t barrier_bytes(const sq_ctx *ctx) {
 //   FP64           41.5  20.1  54.1  26.7  65.4  43.0  68.2  54.2  86.4  78.0
 // (whole solves over their iterations, reliable updates included, at one
 // thread per site then: with a site's directions on four warps, 2048 sites
-// take 9.5 in FP32 and 12.6 in 16-bit, 20736 take 19.2 and 18.0).  With two
+// take 9.5 in FP32 and 12.6 in 16-bit, 20736 take 19.2 and 18.0; FP64 takes 4 %
+// more at 65536 since it compares the neighbours' exponents).  With two
 // rounds per thread it loses: 50.5 against 42.1 at 65536 sites, 170 against
 // 114 at 256000, as the SMs' last round is part empty.
 size_t cg_resident_bytes(const sq_ctx *ctx, int vh, int nrhs, int prec, size_t fb) {

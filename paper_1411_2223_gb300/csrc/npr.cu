@@ -36,7 +36,10 @@
 //   - step 4, four fifths of the work, on the tensor cores: P and Q, at one
 //     scale each, are cut into six signed 9-bit digits, which FP16 holds
 //     exactly, and the digits' products are summed over the 256 (A, C) by
-//     tcgen05.mma into FP32 accumulators in TMEM, exactly (256 256 256 = 2^24).
+//     tcgen05.mma into FP32 accumulators in TMEM, exactly (256 256 256 = 2^24):
+//     the error-free splitting of Ozaki, Ogita, Oishi and Rump ("Error-free
+//     transformations of matrix multiplication by using fast routines of matrix
+//     multiplication and its applications", Numer. Algorithms 59 (2012) 95).
 // A hypercube whose inputs or averaged links do not fit that form (infinities,
 // NaN, elements near the ends of FP64, links far from unitary), or of which an
 // output is so much smaller than the largest products of its P and Q that the
@@ -351,7 +354,7 @@ __global__ void __launch_bounds__(kThreads, 1) npr_fp64_kernel(const NprArgs a) 
 // 15.2 ms with the contraction on the integer units too (three mad.wide.s32
 // per real product, 32 lanes a clock and SM), 9.8 ms with mma.sync (7 thousand
 // cycles per operator, of which ldmatrix reads of the permuted rows 3.7),
-// 8.2 ms here.  About 40 thousand cycles per hypercube go to the steps up to
+// 8.1 ms on tcgen05, 8.3 ms with the comparison below.  About 40 thousand cycles per hypercube go to the steps up to
 // the digits (the integer multiply-adds alone are 10), 5 thousand to each
 // operator: reordering Q, and C from TMEM through shared memory.  Error of a
 // hypercube against long double 3.2e-16 to 3.6e-16, with FP64 FMAs (three per
@@ -881,8 +884,9 @@ __global__ void __launch_bounds__(kFxThreads, 1) npr_kernel(const __grid_constan
     add(a.nops - 1);
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
-  if (sh.fail) {  // the same in every thread; loud, and nothing of it is left running
-    wait_products(done, phase ^ 1);
+  if (sh.fail) {  // the same in every thread: NaN, once the products in flight are
+    // complete or have had eight times the limit more
+    for (int k = 0; k < 8 && !wait_products(done, phase ^ 1); ++k) {}
     if (mine && part < 2)
       for (int op = 0; op < a.nops; ++op) sum[2 * (op * 81 + o) + part] = __longlong_as_double(-1ll);
     for (; h < a.nhc; h += gridDim.x) {
