@@ -119,7 +119,9 @@ typedef struct {
      * and of the D_eo kernel (with the update).  A single system on a lattice of
      * up to 512 sites per parity and SM runs as one resident kernel instead,
      * unless SQ_TUNE_CACHE forces one of these shapes: then its threads per
-     * block and 1.  0 where no batched CG ran. */
+     * block and 1.  (That kernel's blocks run on all SMs at the same time, for
+     * up to 4 ms: it waits for other kernels that fill SMs to end.)  0 where no
+     * batched CG ran. */
     int oe_block, oe_rhs_tile, eo_block, eo_rhs_tile;
 } sq_cg_stats;
 

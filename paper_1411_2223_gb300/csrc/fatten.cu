@@ -169,11 +169,11 @@ __global__ void __launch_bounds__(128) fatten_kernel(FatGeom g, const double2 *u
 // the rows' loads of the same matrices meet in L1.
 //
 // 20^3 x 64, tree-level coefficients: 76.9 ms with a staple kernel per path
-// prefix in FP64 (FP64 units 96 % busy), 8.7 ms here (9.5 ms before the
+// prefix in FP64 (FP64 units 96 % busy), 8.8 ms here (9.5 ms before the
 // products were written as mad.wide.s32, 16.4 ms with a thread per site, which
 // spilled).  The integer multiply-adds alone are 3.2 ms, the fields' traffic
-// 1.9 ms of HBM time; the level-2 kernel issues 3790 instructions per warp for
-// 930 of them and keeps that pipe 57 % busy.  Error against long double 7.6e-17
+// 1.9 ms of HBM time; the level-2 kernel issues 3830 instructions per warp for
+// 930 of them and keeps that pipe 58 % busy.  Error against long double 7.6e-17
 // (before: 2.8e-16), with only the seven-link paths 7.8e-17 (1.5e-16).
 
 struct FatScale {
@@ -392,8 +392,8 @@ __device__ __forceinline__ void row_staple(const AsqtadArgs &a, const SlabSite &
 __device__ __forceinline__ int other_dir(int mu, int k) { return k < mu ? k : k + 1; }
 
 // Are all links unitary?  |U U^dag - 1| < 2^-9 in the parts of every element,
-// which NaN and infinities fail.  Bound by the links' loads (295 MB at 20^3 x 64,
-// 44 us of the 8.7 ms).
+// which NaN and infinities fail.  Bound by the links' loads (76 MB at 16^3 x 32 in
+// 22.5 us, 1 % of a call).
 __global__ void __launch_bounds__(256) fat_scale_kernel(const double2 *u, long nlinks, FatScale *sc) {
   bool even = true;
   for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nlinks;

@@ -36,9 +36,9 @@
 // where every site is computed again (k = 1; with FP64 FMAs 867 for any vector).
 //
 // What it bounds: the FP64 Dslash of one system at 20^3 x 64 went from
-// 321.6 us (FP64 units 100 % busy) to 110 us, 0.84 of the HBM rate for its
+// 321.6 us (FP64 units 100 % busy) to 111 us, 0.82 of the HBM rate for its
 // 2400 bytes per site; with 12 systems, where the links are read once, from
-// 3550 to 999 us (350 instructions per hop and system, 16 warps per SM: bound
+// 3550 to 1010 us (350 instructions per hop and system, 16 warps per SM: bound
 // by their latency).
 #pragma once
 
